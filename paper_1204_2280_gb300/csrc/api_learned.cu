@@ -18,6 +18,8 @@ struct bonsai_mlp {
     int device = 0;
     cudaStream_t stream = nullptr;
     float *P = nullptr, *norm = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr, *loss = nullptr;
+    double *stats = nullptr;       // STATS_BLOCKS x MLP_NNORM block sums of the normalisation
+    unsigned *arrived = nullptr;   // their blocks that have finished
     uint32_t *idx = nullptr;
     long long idx_cap = 0;
     int step = 0;
@@ -171,7 +173,9 @@ int bonsai_mlp_create(bonsai_mlp **out, unsigned long long seed) {
     cudaError_t e = cudaGetDevice(&m->device);
     if (e == cudaSuccess) e = cudaStreamCreate(&m->stream);
     float *buf = nullptr;
-    const size_t total = 4 * (size_t)MLP_NPARAM + MLP_NNORM + 1;
+    const size_t used = 4 * (size_t)MLP_NPARAM + MLP_NNORM + 2;   // parameters, AdamW state, norm, loss, arrivals
+    const size_t stats_off = (used + 1) / 2 * 2;                  // the double sums after them
+    const size_t total = stats_off + 2 * (size_t)STATS_BLOCKS * MLP_NNORM;
     if (e == cudaSuccess) e = cudaMalloc(&buf, total * sizeof(float));
     if (e != cudaSuccess) {
         if (m->stream) cudaStreamDestroy(m->stream);
@@ -181,9 +185,11 @@ int bonsai_mlp_create(bonsai_mlp **out, unsigned long long seed) {
     }
     m->P = buf; m->grad = buf + MLP_NPARAM; m->m = buf + 2 * MLP_NPARAM; m->v = buf + 3 * MLP_NPARAM;
     m->norm = buf + 4 * MLP_NPARAM; m->loss = m->norm + MLP_NNORM;
+    m->arrived = reinterpret_cast<unsigned *>(m->loss + 1);
+    m->stats = reinterpret_cast<double *>(buf + stats_off);
     // He-normal weights (std sqrt(2 / fan_in)), zero biases, identity
     // normalisation.
-    std::vector<float> h(total, 0.f);
+    std::vector<float> h(used, 0.f);
     Rng r(seed);
     const int fan[3] = {MLP_IN, MLP_H, MLP_H}, rows[3] = {MLP_H, MLP_H, MLP_OUT};
     int off = 0;
@@ -194,7 +200,7 @@ int bonsai_mlp_create(bonsai_mlp **out, unsigned long long seed) {
     }
     for (int k = 0; k < MLP_IN; k++) h[4 * MLP_NPARAM + MLP_IN + k] = 1.f;
     h[4 * MLP_NPARAM + 2 * MLP_IN] = 1.f;
-    e = cudaMemcpy(buf, h.data(), total * sizeof(float), cudaMemcpyHostToDevice);
+    e = cudaMemcpy(buf, h.data(), used * sizeof(float), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { bonsai_mlp_destroy(m); cudaGetLastError(); return BONSAI_ERR_CUDA; }
     *out = m;
     return BONSAI_OK;
@@ -231,7 +237,7 @@ int bonsai_mlp_fit_norm(bonsai_mlp *m, const float *X, const float *Y, long long
     DevView dx, dy;
     MCK(to_device(dx, X, (size_t)n * MLP_IN, on_device, m->stream));
     MCK(to_device(dy, Y, (size_t)n * MLP_OUT, on_device, m->stream));
-    MCK(launch_feature_stats(m->stream, dx.p, dy.p, (int)n, m->norm));
+    MCK(launch_feature_stats(m->stream, dx.p, dy.p, (int)n, m->stats, m->arrived, m->norm));
     MCK(cudaStreamSynchronize(m->stream));
     m->fitted = true;
     return BONSAI_OK;
@@ -258,14 +264,9 @@ int bonsai_mlp_grad(bonsai_mlp *m, const float *X, const float *Y, long long n, 
     DevView dx, dy;
     MCK(to_device(dx, X, (size_t)n * MLP_IN, on_device, m->stream));
     MCK(to_device(dy, Y, (size_t)n * MLP_OUT, on_device, m->stream));
-    int r = ensure_idx(m, n);
-    if (r) return r;
-    std::vector<uint32_t> id((size_t)n);
-    for (long long i = 0; i < n; i++) id[(size_t)i] = (uint32_t)i;
-    MCK(cudaMemcpyAsync(m->idx, id.data(), sizeof(uint32_t) * (size_t)n, cudaMemcpyHostToDevice, m->stream));
     MCK(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), m->stream));
     MCK(cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
-    MCK(launch_mlp_grad(m->stream, m->P, m->norm, dx.p, dy.p, m->idx, (int)n, m->grad, m->loss));
+    MCK(launch_mlp_grad(m->stream, m->P, m->norm, dx.p, dy.p, nullptr, (int)n, m->grad, m->loss));
     if (grad) MCK(cudaMemcpyAsync(grad, m->grad, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     if (loss) MCK(cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     MCK(cudaStreamSynchronize(m->stream));
@@ -280,7 +281,7 @@ int bonsai_mlp_train(bonsai_mlp *m, const float *X, const float *Y, long long n,
     MCK(to_device(dx, X, (size_t)n * MLP_IN, on_device, m->stream));
     MCK(to_device(dy, Y, (size_t)n * MLP_OUT, on_device, m->stream));
     if (!m->fitted) {
-        MCK(launch_feature_stats(m->stream, dx.p, dy.p, (int)n, m->norm));
+        MCK(launch_feature_stats(m->stream, dx.p, dy.p, (int)n, m->stats, m->arrived, m->norm));
         m->fitted = true;
     }
     int r = ensure_idx(m, n);
@@ -289,6 +290,8 @@ int bonsai_mlp_train(bonsai_mlp *m, const float *X, const float *Y, long long n,
     std::vector<uint32_t> perm((size_t)n);
     for (long long i = 0; i < n; i++) perm[(size_t)i] = (uint32_t)i;
     const long long nb = (n + batch - 1) / batch;
+    // zero for the first batch; each update clears it for the next
+    MCK(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), m->stream));
     for (int ep = 0; ep < epochs; ep++) {
         for (long long i = n - 1; i > 0; i--) {               // Fisher-Yates
             const long long j = (long long)(rng.next() % (unsigned long long)(i + 1));
@@ -298,7 +301,6 @@ int bonsai_mlp_train(bonsai_mlp *m, const float *X, const float *Y, long long n,
         MCK(cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
         for (long long b = 0; b < nb; b++) {
             const int bsz = (int)std::min<long long>(batch, n - b * batch);
-            MCK(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), m->stream));
             MCK(launch_mlp_grad(m->stream, m->P, m->norm, dx.p, dy.p, m->idx + b * batch, bsz, m->grad, m->loss));
             MCK(launch_adamw(m->stream, m->P, m->grad, m->m, m->v, lr, wd, ++m->step));
         }

@@ -8,9 +8,9 @@
 // BF16, products accumulated in FP32, biases FP32.  Inference runs on the
 // tensor cores (mma.sync m16n8k16, BF16 x BF16 -> FP32; the accumulator
 // layout of one layer is the A-fragment layout of the next, so activations
-// never leave registers).  Training: one thread per sample for forward and
-// backward in FP32 on the same BF16-rounded values, warp-reduced gradients,
-// AdamW on FP32 master weights.
+// never leave registers).  Training: forward and backward of 32-sample tiles
+// in FP32 on the same BF16-rounded values, gradients in registers, AdamW on
+// FP32 master weights.
 //
 // The correction is rotation-equivariant: the 12 inputs are invariants of
 // the body (log|a_tree|, log(-phi_tree), log(1 + accepted cells) in the level
@@ -23,6 +23,7 @@
 // o is parallel to e0 or zero), e2 = e0 x e1.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -263,114 +264,218 @@ k_mlp_rows(const float *__restrict__ P, const float *__restrict__ norm, const fl
 }
 
 // ---------------------------------------------------------------------------
-// Training: forward + backward, one thread per sample.
+// Training: forward + backward of tiles of 32 samples per block.
+//
+// Bound: FP32 issue and shared-memory wavefronts.  A tile is five small
+// products (units x samples forward and backward, units x units for the
+// gradient of W2); each thread holds a register tile of 4 units x 2 samples
+// (4 x 4 parameters for the gradient of W2), so that one 16-byte broadcast
+// and one 8-byte read feed eight multiply-adds and both pipes take about as
+// long (some 3600 cycles a tile each way).  32 samples a tile: a batch of
+// 4096 is 128 blocks, one per SM.  One thread per sample with whole
+// activation vectors in local memory and a five-step warp reduction and
+// shared atomic per parameter took 956 us for a batch of 4096; this takes
+// 27 us (both from a cold cache, without the launch gap).
+//
+// Every activation and every back-propagated value is one chain of fused
+// multiply-adds over its inputs in index order, so it does not depend on the
+// tiling; the parameter gradients are summed over the tile's samples in
+// registers, across the tiles of a block, then with one atomic per parameter
+// and block.
 // ---------------------------------------------------------------------------
 constexpr int TR_THREADS = 256;
+constexpr int TR_S = 32;          // samples per tile (two per thread, 16 threads across)
+constexpr int TR_LD = 36;         // row stride of the sample-major arrays: 16 rows apart read without conflicts
+constexpr int TR_W2T = MLP_H + 4; // row stride of the transposed W2
 
-struct TrShared {
-    float w[MLP_NPARAM];      // BF16-rounded weights (biases exact)
-    float g[MLP_NPARAM];      // block gradient sums
+struct __align__(16) TrShared {
+    float w1t[MLP_IN][MLP_H];     // BF16-rounded weights; [in][out] for the forward products
+    float w2t[MLP_H][TR_W2T];
+    float w2[MLP_H][MLP_H];       // [out][in] for the backward product
+    float w3[MLP_OUT][MLP_H];
+    float b1[MLP_H], b2[MLP_H], b3[4];
+    float x[MLP_IN][TR_LD];       // [unit][sample]
+    float h1[MLP_H][TR_LD], h2[MLP_H][TR_LD], d2[MLP_H][TR_LD], d1[MLP_H][TR_LD];
+    float dy[MLP_OUT][TR_LD];
+    uint32_t row[TR_S];
     float loss;
 };
 
+// acc[u][s] <- chain over k of w[k][j0 + u] * in[k][s0 + s], k ascending.
+template <int K, int LDW>
+__device__ __forceinline__ void tile42(const float *w, const float *in, int j0, int s0, float (&acc)[4][2]) {
+#pragma unroll 8
+    for (int k = 0; k < K; k++) {
+        const float4 a = *reinterpret_cast<const float4 *>(w + k * LDW + j0);
+        const float2 b = *reinterpret_cast<const float2 *>(in + k * TR_LD + s0);
+        acc[0][0] = fmaf(a.x, b.x, acc[0][0]); acc[0][1] = fmaf(a.x, b.y, acc[0][1]);
+        acc[1][0] = fmaf(a.y, b.x, acc[1][0]); acc[1][1] = fmaf(a.y, b.y, acc[1][1]);
+        acc[2][0] = fmaf(a.z, b.x, acc[2][0]); acc[2][1] = fmaf(a.z, b.y, acc[2][1]);
+        acc[3][0] = fmaf(a.w, b.x, acc[3][0]); acc[3][1] = fmaf(a.w, b.y, acc[3][1]);
+    }
+}
+
+// Sum over the tile's samples of a[s] * b[s], added to acc in sample order.
+__device__ __forceinline__ float dot_rows(const float *a, const float *b, float acc) {
+#pragma unroll
+    for (int s = 0; s < TR_S; s += 4) {
+        const float4 u = *reinterpret_cast<const float4 *>(a + s), v = *reinterpret_cast<const float4 *>(b + s);
+        acc = fmaf(u.x, v.x, acc); acc = fmaf(u.y, v.y, acc);
+        acc = fmaf(u.z, v.z, acc); acc = fmaf(u.w, v.w, acc);
+    }
+    return acc;
+}
+
+__device__ __forceinline__ float sum_row(const float *a, float acc) {
+#pragma unroll
+    for (int s = 0; s < TR_S; s += 4) {
+        const float4 u = *reinterpret_cast<const float4 *>(a + s);
+        acc += u.x; acc += u.y; acc += u.z; acc += u.w;
+    }
+    return acc;
+}
+
 // X: n x 12 raw features, Y: n x 3 targets (divided by ysig here), idx:
-// the samples of this batch.  grad += d(loss)/dP with loss = mean over the
-// batch and the 3 outputs of the squared error.
-__global__ void __launch_bounds__(TR_THREADS)
+// the samples of this batch (NULL: rows 0..bsz-1).  grad += d(loss)/dP with
+// loss = mean over the batch and the 3 outputs of the squared error.
+__global__ void __launch_bounds__(TR_THREADS, 2)
 k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const float *__restrict__ X,
            const float *__restrict__ Y, const uint32_t *__restrict__ idx, int bsz, float *grad,
            float *loss) {
-    extern __shared__ float smem_f[];
-    TrShared &S = *reinterpret_cast<TrShared *>(smem_f);
-    const int tid = threadIdx.x, lane = tid & 31;
-    for (int i = tid; i < MLP_NPARAM; i += blockDim.x) {
-        const bool bias = (i >= OFF_B1 && i < OFF_W2) || (i >= OFF_B2 && i < OFF_W3) || i >= OFF_B3;
-        S.w[i] = bias ? P[i] : bf16r(P[i]);
-        S.g[i] = 0.f;
+    extern __shared__ float4 smem_tr[];
+    TrShared &S = *reinterpret_cast<TrShared *>(smem_tr);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < MLP_H * MLP_IN; i += TR_THREADS) S.w1t[i % MLP_IN][i / MLP_IN] = bf16r(P[OFF_W1 + i]);
+    for (int i = tid; i < MLP_H * MLP_H; i += TR_THREADS) {
+        const float v = bf16r(P[OFF_W2 + i]);
+        S.w2[i / MLP_H][i % MLP_H] = v;
+        S.w2t[i % MLP_H][i / MLP_H] = v;
     }
+    if (tid < MLP_OUT * MLP_H) S.w3[tid / MLP_H][tid % MLP_H] = bf16r(P[OFF_W3 + tid]);
+    if (tid < MLP_H) { S.b1[tid] = P[OFF_B1 + tid]; S.b2[tid] = P[OFF_B2 + tid]; }
+    if (tid < MLP_OUT) S.b3[tid] = P[OFF_B3 + tid];
     if (tid == 0) S.loss = 0.f;
+
+    const int j0 = 8 * warp + 4 * (lane >> 4), s0 = 2 * (lane & 15);   // 4 units x 2 samples
+    const int gi = lane & 15, gj = 2 * warp + (lane >> 4);             // W2 parameters (gj + 16 a, gi + 16 b)
+    const int wj = tid & (MLP_H - 1), wi = tid >> 6;                   // W1 parameters (wj, wi + 4 k)
+    float g2[4][4], g1[3] = {0.f, 0.f, 0.f}, g3 = 0.f, gb = 0.f, l = 0.f;
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) g2[a][b] = 0.f;
+    const float sc = 2.f / (3.f * (float)bsz), ysig = norm[2 * MLP_IN];
+
+    for (int t0 = blockIdx.x * TR_S; t0 < bsz; t0 += gridDim.x * TR_S) {
+        if (tid < TR_S) {
+            const int k = t0 + tid;
+            S.row[tid] = k < bsz ? (idx ? idx[k] : (uint32_t)k) : 0xffffffffu;
+        }
+        __syncthreads();
+        for (int e = tid; e < TR_S * MLP_IN; e += TR_THREADS) {
+            const int s = e / MLP_IN, i = e % MLP_IN;
+            const uint32_t r = S.row[s];
+            S.x[i][s] = r != 0xffffffffu ? bf16r((X[(size_t)r * MLP_IN + i] - norm[i]) / norm[MLP_IN + i]) : 0.f;
+        }
+        __syncthreads();
+        float v[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u][0] = v[u][1] = S.b1[j0 + u];
+        tile42<MLP_IN, MLP_H>(&S.w1t[0][0], &S.x[0][0], j0, s0, v);
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            *reinterpret_cast<float2 *>(&S.h1[j0 + u][s0]) =
+                make_float2(bf16r(fmaxf(v[u][0], 0.f)), bf16r(fmaxf(v[u][1], 0.f)));
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u][0] = v[u][1] = S.b2[j0 + u];
+        tile42<MLP_H, TR_W2T>(&S.w2t[0][0], &S.h1[0][0], j0, s0, v);
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            *reinterpret_cast<float2 *>(&S.h2[j0 + u][s0]) =
+                make_float2(bf16r(fmaxf(v[u][0], 0.f)), bf16r(fmaxf(v[u][1], 0.f)));
+        __syncthreads();
+        if (warp < MLP_OUT) {                      // outputs: warp = output, lane = sample
+            float o = S.b3[warp];
+#pragma unroll 16
+            for (int i = 0; i < MLP_H; i++) o = fmaf(S.w3[warp][i], S.h2[i][lane], o);
+            const uint32_t r = S.row[lane];
+            const float res = r != 0xffffffffu ? o - Y[(size_t)r * MLP_OUT + warp] / ysig : 0.f;
+            l += res * res;
+            S.dy[warp][lane] = sc * res;
+        }
+        __syncthreads();
+        // Backward: d2 = W3^T dy (ReLU gate), d1 = W2^T d2 (ReLU gate).
+        for (int i = warp; i < MLP_H; i += TR_THREADS / 32) {
+            float d = 0.f;
+#pragma unroll
+            for (int o = 0; o < MLP_OUT; o++) d = fmaf(S.w3[o][i], S.dy[o][lane], d);
+            S.d2[i][lane] = S.h2[i][lane] > 0.f ? d : 0.f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u][0] = v[u][1] = 0.f;
+        tile42<MLP_H, MLP_H>(&S.w2[0][0], &S.d2[0][0], j0, s0, v);
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const float2 h = *reinterpret_cast<const float2 *>(&S.h1[j0 + u][s0]);
+            *reinterpret_cast<float2 *>(&S.d1[j0 + u][s0]) =
+                make_float2(h.x > 0.f ? v[u][0] : 0.f, h.y > 0.f ? v[u][1] : 0.f);
+        }
+        // Gradients of W2, W3 and the last two biases (need no d1).
+#pragma unroll 2
+        for (int s = 0; s < TR_S; s += 4) {
+            float4 p[4], q[4];
+#pragma unroll
+            for (int a = 0; a < 4; a++) {
+                p[a] = *reinterpret_cast<const float4 *>(&S.d2[gj + 16 * a][s]);
+                q[a] = *reinterpret_cast<const float4 *>(&S.h1[gi + 16 * a][s]);
+            }
+#pragma unroll
+            for (int a = 0; a < 4; a++)
+#pragma unroll
+                for (int b = 0; b < 4; b++) {
+                    g2[a][b] = fmaf(p[a].x, q[b].x, g2[a][b]); g2[a][b] = fmaf(p[a].y, q[b].y, g2[a][b]);
+                    g2[a][b] = fmaf(p[a].z, q[b].z, g2[a][b]); g2[a][b] = fmaf(p[a].w, q[b].w, g2[a][b]);
+                }
+        }
+        if (tid < MLP_OUT * MLP_H) g3 = dot_rows(S.dy[tid / MLP_H], S.h2[tid % MLP_H], g3);
+        if (tid < MLP_H) gb = sum_row(S.d2[tid], gb);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 3; k++) g1[k] = dot_rows(S.d1[wj], S.x[wi + 4 * k], g1[k]);
+        if (tid >= MLP_H && tid < 2 * MLP_H) gb = sum_row(S.d1[tid - MLP_H], gb);
+        if (tid >= 2 * MLP_H && tid < 2 * MLP_H + MLP_OUT) gb = sum_row(S.dy[tid - 2 * MLP_H], gb);
+        __syncthreads();                            // the arrays are rewritten by the next tile
+    }
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) atomicAdd(&grad[OFF_W2 + (gj + 16 * a) * MLP_H + gi + 16 * b], g2[a][b]);
+#pragma unroll
+    for (int k = 0; k < 3; k++) atomicAdd(&grad[OFF_W1 + wj * MLP_IN + wi + 4 * k], g1[k]);
+    if (tid < MLP_OUT * MLP_H) atomicAdd(&grad[OFF_W3 + tid], g3);
+    if (tid < MLP_H) atomicAdd(&grad[OFF_B2 + tid], gb);
+    else if (tid < 2 * MLP_H) atomicAdd(&grad[OFF_B1 + tid - MLP_H], gb);
+    else if (tid < 2 * MLP_H + MLP_OUT) atomicAdd(&grad[OFF_B3 + tid - 2 * MLP_H], gb);
+    if (warp < MLP_OUT) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) atomicAdd(&S.loss, l);
+    }
     __syncthreads();
-    const int k = blockIdx.x * blockDim.x + tid;
-    const bool live = k < bsz;
-    const uint32_t sidx = live ? idx[k] : 0u;
-    float x[MLP_IN];
-#pragma unroll
-    for (int i = 0; i < MLP_IN; i++)
-        x[i] = live ? bf16r((X[(size_t)sidx * MLP_IN + i] - norm[i]) / norm[MLP_IN + i]) : 0.f;
-    float h1[MLP_H], h2[MLP_H];
-    for (int j = 0; j < MLP_H; j++) {
-        float s = S.w[OFF_B1 + j];
-#pragma unroll
-        for (int i = 0; i < MLP_IN; i++) s = fmaf(S.w[OFF_W1 + j * MLP_IN + i], x[i], s);
-        h1[j] = bf16r(fmaxf(s, 0.f));
-    }
-    for (int j = 0; j < MLP_H; j++) {
-        float s = S.w[OFF_B2 + j];
-        for (int i = 0; i < MLP_H; i++) s = fmaf(S.w[OFF_W2 + j * MLP_H + i], h1[i], s);
-        h2[j] = bf16r(fmaxf(s, 0.f));
-    }
-    float dy[MLP_OUT];
-    float l = 0.f;
-    const float sc = 2.f / (3.f * (float)bsz);
-#pragma unroll
-    for (int o = 0; o < MLP_OUT; o++) {
-        float s = S.w[OFF_B3 + o];
-        for (int i = 0; i < MLP_H; i++) s = fmaf(S.w[OFF_W3 + o * MLP_H + i], h2[i], s);
-        const float r = live ? s - Y[(size_t)sidx * MLP_OUT + o] / norm[2 * MLP_IN] : 0.f;
-        l += r * r;
-        dy[o] = sc * r;
-    }
-    // Backward: dh2 = W3^T dy (ReLU gate), dh1 = W2^T dh2 (ReLU gate).
-    float dh2[MLP_H];
-    for (int i = 0; i < MLP_H; i++) {
-        float s = 0.f;
-#pragma unroll
-        for (int o = 0; o < MLP_OUT; o++) s = fmaf(S.w[OFF_W3 + o * MLP_H + i], dy[o], s);
-        dh2[i] = h2[i] > 0.f ? s : 0.f;
-    }
-    float dh1[MLP_H];
-    for (int i = 0; i < MLP_H; i++) {
-        float s = 0.f;
-        for (int j = 0; j < MLP_H; j++) s = fmaf(S.w[OFF_W2 + j * MLP_H + i], dh2[j], s);
-        dh1[i] = h1[i] > 0.f ? s : 0.f;
-    }
-    // Warp-reduced parameter gradients, then shared, then global.
-    auto put = [&](int p, float v) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) atomicAdd(&S.g[p], v);
-    };
-    for (int o = 0; o < MLP_OUT; o++) {
-        put(OFF_B3 + o, dy[o]);
-        for (int i = 0; i < MLP_H; i++) put(OFF_W3 + o * MLP_H + i, dy[o] * h2[i]);
-    }
-    for (int j = 0; j < MLP_H; j++) {
-        put(OFF_B2 + j, dh2[j]);
-        for (int i = 0; i < MLP_H; i++) put(OFF_W2 + j * MLP_H + i, dh2[j] * h1[i]);
-    }
-    for (int j = 0; j < MLP_H; j++) {
-        put(OFF_B1 + j, dh1[j]);
-#pragma unroll
-        for (int i = 0; i < MLP_IN; i++) put(OFF_W1 + j * MLP_IN + i, dh1[j] * x[i]);
-    }
-    {
-        float v = l;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) atomicAdd(&S.loss, v);
-    }
-    __syncthreads();
-    for (int i = tid; i < MLP_NPARAM; i += blockDim.x) atomicAdd(&grad[i], S.g[i]);
     if (tid == 0) atomicAdd(loss, S.loss / (3.f * (float)bsz));
 }
 
 // AdamW (decoupled weight decay on the weight matrices, not the biases).
-__global__ void k_adamw(float *P, const float *__restrict__ grad, float *m, float *v, float lr, float b1,
+// Leaves the gradient at zero for the next batch's sums.
+__global__ void k_adamw(float *P, float *grad, float *m, float *v, float lr, float b1,
                         float b2, float eps, float wd, float bc1, float bc2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MLP_NPARAM) return;
     const bool bias = (i >= OFF_B1 && i < OFF_W2) || (i >= OFF_B2 && i < OFF_W3) || i >= OFF_B3;
     const float g = grad[i];
+    grad[i] = 0.f;
     const float mi = b1 * m[i] + (1.f - b1) * g;
     const float vi = b2 * v[i] + (1.f - b2) * g * g;
     m[i] = mi;
@@ -402,11 +507,16 @@ cudaError_t launch_mlp_grad(cudaStream_t s, const float *P, const float *norm, c
     const size_t smem = sizeof(TrShared);
     cudaError_t e = allow_dyn_smem((const void *)k_mlp_grad, smem, attr_done);
     if (e != cudaSuccess) return e;
-    k_mlp_grad<<<(bsz + TR_THREADS - 1) / TR_THREADS, TR_THREADS, smem, s>>>(P, norm, X, Y, idx, bsz, grad, loss);
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    // two resident blocks per SM; larger batches loop over their tiles
+    const int grid = std::min((bsz + TR_S - 1) / TR_S, 2 * sms);
+    k_mlp_grad<<<grid, TR_THREADS, smem, s>>>(P, norm, X, Y, idx, bsz, grad, loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adamw(cudaStream_t s, float *P, const float *grad, float *m, float *v, float lr, float wd,
+cudaError_t launch_adamw(cudaStream_t s, float *P, float *grad, float *m, float *v, float lr, float wd,
                          int step) {
     const float b1 = 0.9f, b2 = 0.999f;
     const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
@@ -459,37 +569,60 @@ cudaError_t launch_labels(Ctx &c, const uint32_t *targets, int ntar, const float
 }
 
 // Input normalisation of a training set: per-feature mean and standard
-// deviation (FP64 sums), and the RMS of the targets.  One block.
-__global__ void __launch_bounds__(1024) k_feature_stats(const float *__restrict__ X, const float *__restrict__ Y,
-                                                        int n, float *norm) {
-    __shared__ double red[32][2 * MLP_IN + 1];
+// deviation (FP64 sums), and the RMS of the targets.  Each block sums its
+// rows (a warp reduction per block, no atomics), the last block to finish
+// adds the blocks' sums in block order.  FP64 adds bound it (1/64 of the
+// FP32 rate), so the rows go over STATS_BLOCKS blocks: 801 us for 65,536
+// rows in one block, 27 us here.
+__global__ void __launch_bounds__(STATS_THREADS)
+k_feature_stats(const float *__restrict__ X, const float *__restrict__ Y, int n, double *part, unsigned *arrived,
+                float *norm) {
+    constexpr int NV = MLP_NNORM, NW = STATS_THREADS / 32;
+    __shared__ double red[NW][NV];
+    __shared__ bool s_last;
     double s[MLP_IN], q[MLP_IN], yy = 0.0;
+#pragma unroll
     for (int k = 0; k < MLP_IN; k++) { s[k] = 0.0; q[k] = 0.0; }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (long long i = blockIdx.x * STATS_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * STATS_THREADS) {
+#pragma unroll
         for (int k = 0; k < MLP_IN; k++) {
             const double v = X[(size_t)i * MLP_IN + k];
             s[k] += v; q[k] += v * v;
         }
+#pragma unroll
         for (int o = 0; o < MLP_OUT; o++) { const double v = Y[(size_t)i * MLP_OUT + o]; yy += v * v; }
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
     for (int k = 0; k < MLP_IN; k++) {
+#pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
             q[k] += __shfl_xor_sync(0xffffffffu, q[k], o);
         }
+        if (lane == 0) { red[w][k] = s[k]; red[w][MLP_IN + k] = q[k]; }
     }
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) yy += __shfl_xor_sync(0xffffffffu, yy, o);
-    if (lane == 0) {
-        for (int k = 0; k < MLP_IN; k++) { red[w][k] = s[k]; red[w][MLP_IN + k] = q[k]; }
-        red[w][2 * MLP_IN] = yy;
+    if (lane == 0) red[w][2 * MLP_IN] = yy;
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double t = 0.0;
+        for (int j = 0; j < NW; j++) t += red[j][threadIdx.x];
+        part[(size_t)blockIdx.x * NV + threadIdx.x] = t;
+        __threadfence();
     }
     __syncthreads();
-    if (threadIdx.x < 2 * MLP_IN + 1) {
+    if (threadIdx.x == 0) s_last = atomicAdd(arrived, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x < NV) {
         double t = 0.0;
-        for (int j = 0; j < (int)(blockDim.x >> 5); j++) t += red[j][threadIdx.x];
+        for (unsigned j = 0; j < gridDim.x; j++) t += __ldcg(part + (size_t)j * NV + threadIdx.x);
         red[0][threadIdx.x] = t;
     }
+    if (threadIdx.x == 0) *arrived = 0u;
     __syncthreads();
     if (threadIdx.x < MLP_IN) {
         const int k = threadIdx.x;
@@ -500,8 +633,10 @@ __global__ void __launch_bounds__(1024) k_feature_stats(const float *__restrict_
     if (threadIdx.x == 0) norm[2 * MLP_IN] = (float)fmax(sqrt(red[0][2 * MLP_IN] / (3.0 * n)), 1e-12);
 }
 
-cudaError_t launch_feature_stats(cudaStream_t s, const float *X, const float *Y, int n, float *norm) {
-    k_feature_stats<<<1, 1024, 0, s>>>(X, Y, n, norm);
+cudaError_t launch_feature_stats(cudaStream_t s, const float *X, const float *Y, int n, double *part,
+                                 unsigned *arrived, float *norm) {
+    const int grid = std::min((n + STATS_THREADS - 1) / STATS_THREADS, STATS_BLOCKS);
+    k_feature_stats<<<grid, STATS_THREADS, 0, s>>>(X, Y, n, part, arrived, norm);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,46 @@
+"""GPU kernels at the sizes where their tiling, splitting or dispatch changes,
+against the oracle or a plain reference of the same operation."""
+import numpy as np
+import pytest
+
+import paper_1204_2280_gb300 as B
+from oracle import mlp as OM
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 4097, 40000])
+def test_training_gradient_tiles(n):
+    """Gradient and loss of n rows (32-row tiles, up to 304 blocks that loop
+    over them) against the FP64 oracle on the same BF16-rounded values.  An
+    activation within FP32 rounding of a BF16 tie may round the other way
+    (2^-8 of one activation), so the gradient is held to 2^-6 of its norm and
+    the loss to 2^-8."""
+    rng = np.random.default_rng(n)
+    X = rng.normal(size=(n, B.MLP_IN)).astype(np.float32)
+    Y = (rng.normal(size=(n, B.MLP_OUT)) * 5e-3).astype(np.float32)
+    net = B.MLP(3)
+    norm = np.concatenate([np.zeros(B.MLP_IN), np.ones(B.MLP_IN), [5e-3]]).astype(np.float32)
+    net.set_params(None, norm)
+    P, _ = net.get_params()
+    g, loss = net.grad(X, Y)
+    loss_ref, g_ref = OM.loss_grad(P, norm, X, Y)
+    assert np.linalg.norm(g - g_ref) <= 2.0 ** -6 * np.linalg.norm(g_ref)
+    assert abs(loss - loss_ref) <= 2.0 ** -8 * loss_ref
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 152 * 128 + 1])
+def test_normalisation_blocks(n):
+    """Mean, standard deviation and target RMS over one to all blocks: FP64
+    sums, so FP32 results within one rounding of numpy's (the standard
+    deviation within sqrt of the FP64 cancellation, far below 1e-6 here)."""
+    rng = np.random.default_rng(n)
+    X = (rng.normal(size=(n, B.MLP_IN)) + 2.0).astype(np.float32)
+    Y = rng.normal(size=(n, B.MLP_OUT)).astype(np.float32)
+    net = B.MLP(0)
+    for _ in range(2):                       # the arrival count starts over
+        net.fit_norm(X, Y)
+        _, norm = net.get_params()
+        x, y = X.astype(np.float64), Y.astype(np.float64)
+        ref = np.concatenate([x.mean(0), np.maximum(x.std(0), 1e-6), [np.sqrt((y * y).mean())]])
+        assert np.abs(norm - ref).max() <= 1e-6 * np.abs(ref).max()
