@@ -275,7 +275,8 @@ k_mlp_rows(const float *__restrict__ P, const float *__restrict__ norm, const fl
 // 4096 is 128 blocks, one per SM.  One thread per sample with whole
 // activation vectors in local memory and a five-step warp reduction and
 // shared atomic per parameter took 956 us for a batch of 4096; this takes
-// 27 us (both from a cold cache, without the launch gap).
+// 20 us (both from a cold cache, without the launch gap; 27 us before inputs
+// were fetched a tile ahead and the weights staged in one round trip).
 //
 // Every activation and every back-propagated value is one chain of fused
 // multiply-adds over its inputs in index order, so it does not depend on the
@@ -294,12 +295,14 @@ struct __align__(16) TrShared {
     float w2[MLP_H][MLP_H];       // [out][in] for the backward product
     float w3[MLP_OUT][MLP_H];
     float b1[MLP_H], b2[MLP_H], b3[4];
+    float norm[2 * MLP_IN];
     float x[MLP_IN][TR_LD];       // [unit][sample]
     float h1[MLP_H][TR_LD], h2[MLP_H][TR_LD], d2[MLP_H][TR_LD], d1[MLP_H][TR_LD];
     float dy[MLP_OUT][TR_LD];
-    uint32_t row[TR_S];
     float loss;
 };
+static_assert(MLP_H * MLP_H % TR_THREADS == 0 && MLP_H * MLP_IN % TR_THREADS == 0, "weights staged in whole rounds");
+static_assert(TR_S * MLP_IN <= 2 * TR_THREADS && TR_THREADS >= 32 * MLP_OUT, "a tile's inputs are two per thread");
 
 // acc[u][s] <- chain over k of w[k][j0 + u] * in[k][s0 + s], k ascending.
 template <int K, int LDW>
@@ -345,16 +348,49 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
     extern __shared__ float4 smem_tr[];
     TrShared &S = *reinterpret_cast<TrShared *>(smem_tr);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < MLP_H * MLP_IN; i += TR_THREADS) S.w1t[i % MLP_IN][i / MLP_IN] = bf16r(P[OFF_W1 + i]);
-    for (int i = tid; i < MLP_H * MLP_H; i += TR_THREADS) {
-        const float v = bf16r(P[OFF_W2 + i]);
-        S.w2[i / MLP_H][i % MLP_H] = v;
-        S.w2t[i % MLP_H][i / MLP_H] = v;
+    // This thread's raw inputs (two of the tile's 384) and target of a tile,
+    // fetched a tile ahead: their two dependent round trips (index, row)
+    // overlap the weights' staging or the tile before.  NaN-free zeros where
+    // the batch ends.
+    float xr[2] = {0.f, 0.f}, yr = 0.f;
+    bool on = false;
+    auto fetch = [&](int t0) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int e = tid + h * TR_THREADS, k = t0 + e / MLP_IN;
+            if (e < TR_S * MLP_IN && k < bsz) xr[h] = X[(size_t)(idx ? idx[k] : (uint32_t)k) * MLP_IN + e % MLP_IN];
+        }
+        on = t0 + lane < bsz;
+        if (warp < MLP_OUT && on)
+            yr = Y[(size_t)(idx ? idx[t0 + lane] : (uint32_t)(t0 + lane)) * MLP_OUT + warp];
+    };
+    fetch(blockIdx.x * TR_S);
+    {
+        // all loads in flight at once
+        float w2r[MLP_H * MLP_H / TR_THREADS], w1r[MLP_H * MLP_IN / TR_THREADS];
+#pragma unroll
+        for (int r = 0; r < MLP_H * MLP_H / TR_THREADS; r++) w2r[r] = P[OFF_W2 + tid + r * TR_THREADS];
+#pragma unroll
+        for (int r = 0; r < MLP_H * MLP_IN / TR_THREADS; r++) w1r[r] = P[OFF_W1 + tid + r * TR_THREADS];
+        if (tid < MLP_OUT * MLP_H) S.w3[tid / MLP_H][tid % MLP_H] = bf16r(P[OFF_W3 + tid]);
+        if (tid < MLP_H) { S.b1[tid] = P[OFF_B1 + tid]; S.b2[tid] = P[OFF_B2 + tid]; }
+        if (tid < MLP_OUT) S.b3[tid] = P[OFF_B3 + tid];
+        if (tid < 2 * MLP_IN) S.norm[tid] = norm[tid];
+        if (tid == 0) S.loss = 0.f;
+#pragma unroll
+        for (int r = 0; r < MLP_H * MLP_H / TR_THREADS; r++) {
+            const int i = tid + r * TR_THREADS;
+            const float v = bf16r(w2r[r]);
+            S.w2[i / MLP_H][i % MLP_H] = v;
+            S.w2t[i % MLP_H][i / MLP_H] = v;
+        }
+#pragma unroll
+        for (int r = 0; r < MLP_H * MLP_IN / TR_THREADS; r++) {
+            const int i = tid + r * TR_THREADS;
+            S.w1t[i % MLP_IN][i / MLP_IN] = bf16r(w1r[r]);
+        }
     }
-    if (tid < MLP_OUT * MLP_H) S.w3[tid / MLP_H][tid % MLP_H] = bf16r(P[OFF_W3 + tid]);
-    if (tid < MLP_H) { S.b1[tid] = P[OFF_B1 + tid]; S.b2[tid] = P[OFF_B2 + tid]; }
-    if (tid < MLP_OUT) S.b3[tid] = P[OFF_B3 + tid];
-    if (tid == 0) S.loss = 0.f;
+    __syncthreads();
 
     const int j0 = 8 * warp + 4 * (lane >> 4), s0 = 2 * (lane & 15);   // 4 units x 2 samples
     const int gi = lane & 15, gj = 2 * warp + (lane >> 4);             // W2 parameters (gj + 16 a, gi + 16 b)
@@ -367,16 +403,14 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
     const float sc = 2.f / (3.f * (float)bsz), ysig = norm[2 * MLP_IN];
 
     for (int t0 = blockIdx.x * TR_S; t0 < bsz; t0 += gridDim.x * TR_S) {
-        if (tid < TR_S) {
-            const int k = t0 + tid;
-            S.row[tid] = k < bsz ? (idx ? idx[k] : (uint32_t)k) : 0xffffffffu;
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int e = tid + h * TR_THREADS, sm = e / MLP_IN, i = e % MLP_IN;
+            if (e < TR_S * MLP_IN) S.x[i][sm] = t0 + sm < bsz ? bf16r((xr[h] - S.norm[i]) / S.norm[MLP_IN + i]) : 0.f;
         }
-        __syncthreads();
-        for (int e = tid; e < TR_S * MLP_IN; e += TR_THREADS) {
-            const int s = e / MLP_IN, i = e % MLP_IN;
-            const uint32_t r = S.row[s];
-            S.x[i][s] = r != 0xffffffffu ? bf16r((X[(size_t)r * MLP_IN + i] - norm[i]) / norm[MLP_IN + i]) : 0.f;
-        }
+        const float target = yr / ysig;
+        const bool live = on;
+        if (t0 + (int)gridDim.x * TR_S < bsz) fetch(t0 + gridDim.x * TR_S);
         __syncthreads();
         float v[4][2];
 #pragma unroll
@@ -399,8 +433,7 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
             float o = S.b3[warp];
 #pragma unroll 16
             for (int i = 0; i < MLP_H; i++) o = fmaf(S.w3[warp][i], S.h2[i][lane], o);
-            const uint32_t r = S.row[lane];
-            const float res = r != 0xffffffffu ? o - Y[(size_t)r * MLP_OUT + warp] / ysig : 0.f;
+            const float res = live ? o - target : 0.f;
             l += res * res;
             S.dy[warp][lane] = sc * res;
         }
