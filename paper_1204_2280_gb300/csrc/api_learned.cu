@@ -18,6 +18,7 @@ struct bonsai_mlp {
     int device = 0;
     cudaStream_t stream = nullptr;
     float *P = nullptr, *norm = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr, *loss = nullptr;
+    float *part = nullptr;         // TR_BLOCKS x TR_PART block sums of a batch (allocated by the first gradient)
     double *stats = nullptr;       // STATS_BLOCKS x MLP_NNORM block sums of the normalisation
     unsigned *arrived = nullptr;   // their blocks that have finished
     uint32_t *idx = nullptr;
@@ -159,6 +160,11 @@ int ensure_idx(bonsai_mlp *m, long long n) {
     return BONSAI_OK;
 }
 
+int ensure_part(bonsai_mlp *m) {
+    if (!m->part) MCK(cudaMalloc(&m->part, sizeof(float) * (size_t)TR_BLOCKS * TR_PART));
+    return BONSAI_OK;
+}
+
 // Copies host rows to a temporary device buffer when needed.
 struct DevView {
     const float *p = nullptr;
@@ -225,6 +231,7 @@ void bonsai_mlp_destroy(bonsai_mlp *m) {
     if (m->stream) cudaStreamSynchronize(m->stream);
     if (m->P) cudaFree(m->P);
     if (m->idx) cudaFree(m->idx);
+    if (m->part) cudaFree(m->part);
     if (m->stream) cudaStreamDestroy(m->stream);
     delete m;
 }
@@ -278,9 +285,9 @@ int bonsai_mlp_grad(bonsai_mlp *m, const float *X, const float *Y, long long n, 
     DevView dx, dy;
     MCK(to_device(dx, X, (size_t)n * MLP_IN, on_device, m->stream));
     MCK(to_device(dy, Y, (size_t)n * MLP_OUT, on_device, m->stream));
-    MCK(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), m->stream));
-    MCK(cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
-    MCK(launch_mlp_grad(m->stream, m->P, m->norm, dx.p, dy.p, nullptr, (int)n, m->grad, m->loss));
+    const int r = ensure_part(m);
+    if (r) return r;
+    MCK(launch_mlp_grad(m->stream, m->P, m->norm, dx.p, dy.p, nullptr, (int)n, m->part, m->grad, m->loss));
     if (grad) MCK(cudaMemcpyAsync(grad, m->grad, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     if (loss) MCK(cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     MCK(cudaStreamSynchronize(m->stream));
@@ -299,7 +306,7 @@ int bonsai_mlp_train(bonsai_mlp *m, const float *X, const float *Y, long long n,
         m->fitted = true;
     }
     int r = ensure_idx(m, n);
-    if (r) return r;
+    if (r || (r = ensure_part(m))) return r;
     Rng rng(seed);
     // Two host orders: the next epoch's is shuffled from this one's while the
     // device works, and a copy may read its source until the stream has been
@@ -315,8 +322,6 @@ int bonsai_mlp_train(bonsai_mlp *m, const float *X, const float *Y, long long n,
         }
     };
     const long long nb = (n + batch - 1) / batch;
-    // zero for the first batch; each update clears it for the next
-    MCK(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), m->stream));
     shuffle(order[0]);
     for (int ep = 0; ep < epochs; ep++) {
         const std::vector<uint32_t> &cur = order[ep & 1];
@@ -324,8 +329,8 @@ int bonsai_mlp_train(bonsai_mlp *m, const float *X, const float *Y, long long n,
         MCK(cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
         for (long long b = 0; b < nb; b++) {
             const int bsz = (int)std::min<long long>(batch, n - b * batch);
-            MCK(launch_mlp_grad(m->stream, m->P, m->norm, dx.p, dy.p, m->idx + b * batch, bsz, m->grad, m->loss));
-            MCK(launch_adamw(m->stream, m->P, m->grad, m->m, m->v, lr, wd, ++m->step));
+            MCK(launch_mlp_batch(m->stream, m->P, m->norm, dx.p, dy.p, m->idx + b * batch, bsz, m->part, m->m, m->v,
+                                 m->loss, lr, wd, ++m->step));
         }
         if (ep + 1 < epochs) {
             std::vector<uint32_t> &next = order[(ep + 1) & 1];

@@ -46,6 +46,8 @@ constexpr int MAX_SYSTEMS = 256;                       // ensemble: one more pas
 constexpr int MLP_IN = 12, MLP_H = 64, MLP_OUT = 3;    // learned correction 12 -> 64 -> 64 -> 3
 constexpr int MLP_NPARAM = MLP_H * MLP_IN + MLP_H + MLP_H * MLP_H + MLP_H + MLP_OUT * MLP_H + MLP_OUT;
 constexpr int MLP_NNORM = 2 * MLP_IN + 1;              // mu[12], sigma[12], ysig
+constexpr int TR_BLOCKS = 304;                         // training: gradient blocks (two per SM) and the
+constexpr int TR_PART = (MLP_NPARAM + 1 + 31) / 32 * 32;   // floats of a block's sums (gradient, loss)
 constexpr int STATS_BLOCKS = 152, STATS_THREADS = 128;  // normalisation sums: blocks and threads per block
 constexpr int FEAT_STRIDE = 12;                        // walk features per body
 constexpr int JUDGE_MAX = 4096;                        // sampled bodies of the direct-sum judge
@@ -289,9 +291,10 @@ cudaError_t launch_judge(Ctx &c, const uint32_t *targets, int ntar, const float4
 cudaError_t launch_mlp_infer(Ctx &c, const float *P, const float *norm);
 cudaError_t launch_mlp_rows(cudaStream_t s, const float *P, const float *norm, const float *X, float *Y, int n);
 cudaError_t launch_mlp_grad(cudaStream_t s, const float *P, const float *norm, const float *X, const float *Y,
-                            const uint32_t *idx, int bsz, float *grad, float *loss);
-cudaError_t launch_adamw(cudaStream_t s, float *P, float *grad, float *m, float *v, float lr, float wd,
-                         int step);
+                            const uint32_t *idx, int bsz, float *part, float *grad, float *loss);
+cudaError_t launch_mlp_batch(cudaStream_t s, float *P, const float *norm, const float *X, const float *Y,
+                             const uint32_t *idx, int bsz, float *part, float *m, float *v, float *loss, float lr,
+                             float wd, int step);
 cudaError_t launch_gather_features(Ctx &c, const uint32_t *targets, int ntar, float *X, uint32_t *ids);
 cudaError_t launch_labels(Ctx &c, const uint32_t *targets, int ntar, const float4 *direct, float *Y);
 cudaError_t launch_feature_stats(cudaStream_t s, const float *X, const float *Y, int n, double *part,

@@ -275,16 +275,21 @@ k_mlp_rows(const float *__restrict__ P, const float *__restrict__ norm, const fl
 // 4096 is 128 blocks, one per SM.  One thread per sample with whole
 // activation vectors in local memory and a five-step warp reduction and
 // shared atomic per parameter took 956 us for a batch of 4096; this takes
-// 20 us (both from a cold cache, without the launch gap; 27 us before inputs
-// were fetched a tile ahead and the weights staged in one round trip).
+// about 12 us (27 us before inputs were fetched a tile ahead and the weights
+// staged in one round trip, 20 us with an atomic per parameter and block
+// instead of the blocks' own rows of sums; all from a cold cache).  An epoch
+// of 65,536 rows in 16 batches, device time: 265 us, 16.6 a batch.
 //
 // Every activation and every back-propagated value is one chain of fused
 // multiply-adds over its inputs in index order, so it does not depend on the
 // tiling; the parameter gradients are summed over the tile's samples in
-// registers, across the tiles of a block, then with one atomic per parameter
-// and block.
+// registers, across the tiles of a block, then over the blocks in a fixed
+// order by the kernel that uses them.
 // ---------------------------------------------------------------------------
-constexpr int TR_THREADS = 256;
+constexpr int TR_THREADS = 256;                   // (512 with half the register tile: 293 us an epoch, 265 here)
+constexpr int TR_U = MLP_H * 32 / 2 / TR_THREADS; // units of a thread's register tile
+constexpr int TR_GA = 4 * TR_U / 4;               // W2 gradient rows of a thread (of 4 columns)
+constexpr int TR_GJ = MLP_H / TR_GA;              // threads across the rows
 constexpr int TR_S = 32;          // samples per tile (two per thread, 16 threads across)
 constexpr int TR_LD = 36;         // row stride of the sample-major arrays: 16 rows apart read without conflicts
 constexpr int TR_W2T = MLP_H + 4; // row stride of the transposed W2
@@ -299,22 +304,23 @@ struct __align__(16) TrShared {
     float x[MLP_IN][TR_LD];       // [unit][sample]
     float h1[MLP_H][TR_LD], h2[MLP_H][TR_LD], d2[MLP_H][TR_LD], d1[MLP_H][TR_LD];
     float dy[MLP_OUT][TR_LD];
-    float loss;
 };
-static_assert(MLP_H * MLP_H % TR_THREADS == 0 && MLP_H * MLP_IN % TR_THREADS == 0, "weights staged in whole rounds");
+static_assert(TR_U == 4 && MLP_H * MLP_H % TR_THREADS == 0, "16-byte weight reads, W2 staged in whole rounds");
 static_assert(TR_S * MLP_IN <= 2 * TR_THREADS && TR_THREADS >= 32 * MLP_OUT, "a tile's inputs are two per thread");
 
 // acc[u][s] <- chain over k of w[k][j0 + u] * in[k][s0 + s], k ascending.
 template <int K, int LDW>
-__device__ __forceinline__ void tile42(const float *w, const float *in, int j0, int s0, float (&acc)[4][2]) {
+__device__ __forceinline__ void tile_units(const float *w, const float *in, int j0, int s0, float (&acc)[TR_U][2]) {
 #pragma unroll 8
     for (int k = 0; k < K; k++) {
-        const float4 a = *reinterpret_cast<const float4 *>(w + k * LDW + j0);
+        const float4 v = *reinterpret_cast<const float4 *>(w + k * LDW + j0);
+        const float a[TR_U] = {v.x, v.y, v.z, v.w};
         const float2 b = *reinterpret_cast<const float2 *>(in + k * TR_LD + s0);
-        acc[0][0] = fmaf(a.x, b.x, acc[0][0]); acc[0][1] = fmaf(a.x, b.y, acc[0][1]);
-        acc[1][0] = fmaf(a.y, b.x, acc[1][0]); acc[1][1] = fmaf(a.y, b.y, acc[1][1]);
-        acc[2][0] = fmaf(a.z, b.x, acc[2][0]); acc[2][1] = fmaf(a.z, b.y, acc[2][1]);
-        acc[3][0] = fmaf(a.w, b.x, acc[3][0]); acc[3][1] = fmaf(a.w, b.y, acc[3][1]);
+#pragma unroll
+        for (int u = 0; u < TR_U; u++) {
+            acc[u][0] = fmaf(a[u], b.x, acc[u][0]);
+            acc[u][1] = fmaf(a[u], b.y, acc[u][1]);
+        }
     }
 }
 
@@ -339,12 +345,12 @@ __device__ __forceinline__ float sum_row(const float *a, float acc) {
 }
 
 // X: n x 12 raw features, Y: n x 3 targets (divided by ysig here), idx:
-// the samples of this batch (NULL: rows 0..bsz-1).  grad += d(loss)/dP with
-// loss = mean over the batch and the 3 outputs of the squared error.
+// the samples of this batch (NULL: rows 0..bsz-1).  Each block writes its
+// share of d(loss)/dP and of the loss, the mean over the batch and the 3
+// outputs of the squared error, to its row of part.
 __global__ void __launch_bounds__(TR_THREADS, 2)
 k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const float *__restrict__ X,
-           const float *__restrict__ Y, const uint32_t *__restrict__ idx, int bsz, float *grad,
-           float *loss) {
+           const float *__restrict__ Y, const uint32_t *__restrict__ idx, int bsz, float *part) {
     extern __shared__ float4 smem_tr[];
     TrShared &S = *reinterpret_cast<TrShared *>(smem_tr);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -367,16 +373,16 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
     fetch(blockIdx.x * TR_S);
     {
         // all loads in flight at once
-        float w2r[MLP_H * MLP_H / TR_THREADS], w1r[MLP_H * MLP_IN / TR_THREADS];
+        constexpr int W1R = (MLP_H * MLP_IN + TR_THREADS - 1) / TR_THREADS;
+        float w2r[MLP_H * MLP_H / TR_THREADS], w1r[W1R];
 #pragma unroll
         for (int r = 0; r < MLP_H * MLP_H / TR_THREADS; r++) w2r[r] = P[OFF_W2 + tid + r * TR_THREADS];
 #pragma unroll
-        for (int r = 0; r < MLP_H * MLP_IN / TR_THREADS; r++) w1r[r] = P[OFF_W1 + tid + r * TR_THREADS];
+        for (int r = 0; r < W1R; r++) w1r[r] = tid + r * TR_THREADS < MLP_H * MLP_IN ? P[OFF_W1 + tid + r * TR_THREADS] : 0.f;
         if (tid < MLP_OUT * MLP_H) S.w3[tid / MLP_H][tid % MLP_H] = bf16r(P[OFF_W3 + tid]);
         if (tid < MLP_H) { S.b1[tid] = P[OFF_B1 + tid]; S.b2[tid] = P[OFF_B2 + tid]; }
         if (tid < MLP_OUT) S.b3[tid] = P[OFF_B3 + tid];
         if (tid < 2 * MLP_IN) S.norm[tid] = norm[tid];
-        if (tid == 0) S.loss = 0.f;
 #pragma unroll
         for (int r = 0; r < MLP_H * MLP_H / TR_THREADS; r++) {
             const int i = tid + r * TR_THREADS;
@@ -385,19 +391,20 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
             S.w2t[i % MLP_H][i / MLP_H] = v;
         }
 #pragma unroll
-        for (int r = 0; r < MLP_H * MLP_IN / TR_THREADS; r++) {
+        for (int r = 0; r < W1R; r++) {
             const int i = tid + r * TR_THREADS;
-            S.w1t[i % MLP_IN][i / MLP_IN] = bf16r(w1r[r]);
+            if (i < MLP_H * MLP_IN) S.w1t[i % MLP_IN][i / MLP_IN] = bf16r(w1r[r]);
         }
     }
     __syncthreads();
 
-    const int j0 = 8 * warp + 4 * (lane >> 4), s0 = 2 * (lane & 15);   // 4 units x 2 samples
-    const int gi = lane & 15, gj = 2 * warp + (lane >> 4);             // W2 parameters (gj + 16 a, gi + 16 b)
-    const int wj = tid & (MLP_H - 1), wi = tid >> 6;                   // W1 parameters (wj, wi + 4 k)
-    float g2[4][4], g1[3] = {0.f, 0.f, 0.f}, g3 = 0.f, gb = 0.f, l = 0.f;
+    const int j0 = TR_U * (2 * warp + (lane >> 4)), s0 = 2 * (lane & 15);   // TR_U units x 2 samples
+    const int gi = lane & 15, gj = 2 * warp + (lane >> 4);     // W2 parameters (gj + TR_GJ a, gi + 16 b)
+    constexpr int NW1 = (MLP_H * MLP_IN + TR_THREADS - 1) / TR_THREADS;
+    const int wj = tid & (MLP_H - 1), wi = tid >> 6;           // W1 parameters (wj, wi + TR_THREADS / 64 k)
+    float g2[TR_GA][4], g1[NW1] = {}, g3 = 0.f, gb = 0.f, l = 0.f;
 #pragma unroll
-    for (int a = 0; a < 4; a++)
+    for (int a = 0; a < TR_GA; a++)
 #pragma unroll
         for (int b = 0; b < 4; b++) g2[a][b] = 0.f;
     const float sc = 2.f / (3.f * (float)bsz), ysig = norm[2 * MLP_IN];
@@ -412,20 +419,20 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
         const bool live = on;
         if (t0 + (int)gridDim.x * TR_S < bsz) fetch(t0 + gridDim.x * TR_S);
         __syncthreads();
-        float v[4][2];
+        float v[TR_U][2];
 #pragma unroll
-        for (int u = 0; u < 4; u++) v[u][0] = v[u][1] = S.b1[j0 + u];
-        tile42<MLP_IN, MLP_H>(&S.w1t[0][0], &S.x[0][0], j0, s0, v);
+        for (int u = 0; u < TR_U; u++) v[u][0] = v[u][1] = S.b1[j0 + u];
+        tile_units<MLP_IN, MLP_H>(&S.w1t[0][0], &S.x[0][0], j0, s0, v);
 #pragma unroll
-        for (int u = 0; u < 4; u++)
+        for (int u = 0; u < TR_U; u++)
             *reinterpret_cast<float2 *>(&S.h1[j0 + u][s0]) =
                 make_float2(bf16r(fmaxf(v[u][0], 0.f)), bf16r(fmaxf(v[u][1], 0.f)));
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < 4; u++) v[u][0] = v[u][1] = S.b2[j0 + u];
-        tile42<MLP_H, TR_W2T>(&S.w2t[0][0], &S.h1[0][0], j0, s0, v);
+        for (int u = 0; u < TR_U; u++) v[u][0] = v[u][1] = S.b2[j0 + u];
+        tile_units<MLP_H, TR_W2T>(&S.w2t[0][0], &S.h1[0][0], j0, s0, v);
 #pragma unroll
-        for (int u = 0; u < 4; u++)
+        for (int u = 0; u < TR_U; u++)
             *reinterpret_cast<float2 *>(&S.h2[j0 + u][s0]) =
                 make_float2(bf16r(fmaxf(v[u][0], 0.f)), bf16r(fmaxf(v[u][1], 0.f)));
         __syncthreads();
@@ -447,10 +454,10 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
         }
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < 4; u++) v[u][0] = v[u][1] = 0.f;
-        tile42<MLP_H, MLP_H>(&S.w2[0][0], &S.d2[0][0], j0, s0, v);
+        for (int u = 0; u < TR_U; u++) v[u][0] = v[u][1] = 0.f;
+        tile_units<MLP_H, MLP_H>(&S.w2[0][0], &S.d2[0][0], j0, s0, v);
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
+        for (int u = 0; u < TR_U; u++) {
             const float2 h = *reinterpret_cast<const float2 *>(&S.h1[j0 + u][s0]);
             *reinterpret_cast<float2 *>(&S.d1[j0 + u][s0]) =
                 make_float2(h.x > 0.f ? v[u][0] : 0.f, h.y > 0.f ? v[u][1] : 0.f);
@@ -458,57 +465,98 @@ k_mlp_grad(const float *__restrict__ P, const float *__restrict__ norm, const fl
         // Gradients of W2, W3 and the last two biases (need no d1).
 #pragma unroll 2
         for (int s = 0; s < TR_S; s += 4) {
-            float4 p[4], q[4];
+            float4 p[TR_GA], q[4];
 #pragma unroll
-            for (int a = 0; a < 4; a++) {
-                p[a] = *reinterpret_cast<const float4 *>(&S.d2[gj + 16 * a][s]);
-                q[a] = *reinterpret_cast<const float4 *>(&S.h1[gi + 16 * a][s]);
-            }
+            for (int a = 0; a < TR_GA; a++) p[a] = *reinterpret_cast<const float4 *>(&S.d2[gj + TR_GJ * a][s]);
 #pragma unroll
-            for (int a = 0; a < 4; a++)
+            for (int b = 0; b < 4; b++) q[b] = *reinterpret_cast<const float4 *>(&S.h1[gi + 16 * b][s]);
+#pragma unroll
+            for (int a = 0; a < TR_GA; a++)
 #pragma unroll
                 for (int b = 0; b < 4; b++) {
                     g2[a][b] = fmaf(p[a].x, q[b].x, g2[a][b]); g2[a][b] = fmaf(p[a].y, q[b].y, g2[a][b]);
                     g2[a][b] = fmaf(p[a].z, q[b].z, g2[a][b]); g2[a][b] = fmaf(p[a].w, q[b].w, g2[a][b]);
                 }
         }
-        if (tid < MLP_OUT * MLP_H) g3 = dot_rows(S.dy[tid / MLP_H], S.h2[tid % MLP_H], g3);
+        // (the small sums from the last threads down, W1's below from the first up)
+        const int r3 = TR_THREADS - 1 - tid;
+        if (r3 < MLP_OUT * MLP_H) g3 = dot_rows(S.dy[r3 / MLP_H], S.h2[r3 % MLP_H], g3);
         if (tid < MLP_H) gb = sum_row(S.d2[tid], gb);
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 3; k++) g1[k] = dot_rows(S.d1[wj], S.x[wi + 4 * k], g1[k]);
+        for (int k = 0; k < NW1; k++)
+            if (wi + TR_THREADS / MLP_H * k < MLP_IN) g1[k] = dot_rows(S.d1[wj], S.x[wi + TR_THREADS / MLP_H * k], g1[k]);
         if (tid >= MLP_H && tid < 2 * MLP_H) gb = sum_row(S.d1[tid - MLP_H], gb);
         if (tid >= 2 * MLP_H && tid < 2 * MLP_H + MLP_OUT) gb = sum_row(S.dy[tid - 2 * MLP_H], gb);
         __syncthreads();                            // the arrays are rewritten by the next tile
     }
+    // The block's sums, coalesced, for the kernel that adds the blocks up.
+    float *out = part + (size_t)blockIdx.x * TR_PART;
 #pragma unroll
-    for (int a = 0; a < 4; a++)
+    for (int a = 0; a < TR_GA; a++)
 #pragma unroll
-        for (int b = 0; b < 4; b++) atomicAdd(&grad[OFF_W2 + (gj + 16 * a) * MLP_H + gi + 16 * b], g2[a][b]);
+        for (int b = 0; b < 4; b++) out[OFF_W2 + (gj + TR_GJ * a) * MLP_H + gi + 16 * b] = g2[a][b];
 #pragma unroll
-    for (int k = 0; k < 3; k++) atomicAdd(&grad[OFF_W1 + wj * MLP_IN + wi + 4 * k], g1[k]);
-    if (tid < MLP_OUT * MLP_H) atomicAdd(&grad[OFF_W3 + tid], g3);
-    if (tid < MLP_H) atomicAdd(&grad[OFF_B2 + tid], gb);
-    else if (tid < 2 * MLP_H) atomicAdd(&grad[OFF_B1 + tid - MLP_H], gb);
-    else if (tid < 2 * MLP_H + MLP_OUT) atomicAdd(&grad[OFF_B3 + tid - 2 * MLP_H], gb);
+    for (int k = 0; k < NW1; k++)
+        if (wi + TR_THREADS / MLP_H * k < MLP_IN) out[OFF_W1 + wj * MLP_IN + wi + TR_THREADS / MLP_H * k] = g1[k];
+    const int r3 = TR_THREADS - 1 - tid;
+    if (r3 < MLP_OUT * MLP_H) out[OFF_W3 + r3] = g3;
+    if (tid < MLP_H) out[OFF_B2 + tid] = gb;
+    else if (tid < 2 * MLP_H) out[OFF_B1 + tid - MLP_H] = gb;
+    else if (tid < 2 * MLP_H + MLP_OUT) out[OFF_B3 + tid - 2 * MLP_H] = gb;
     if (warp < MLP_OUT) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-        if (lane == 0) atomicAdd(&S.loss, l);
+        if (lane == 0) S.dy[warp][0] = l;
     }
     __syncthreads();
-    if (tid == 0) atomicAdd(loss, S.loss / (3.f * (float)bsz));
+    if (tid == 0) out[MLP_NPARAM] = (S.dy[0][0] + S.dy[1][0] + S.dy[2][0]) / (3.f * (float)bsz);
 }
 
-// AdamW (decoupled weight decay on the weight matrices, not the biases).
-// Leaves the gradient at zero for the next batch's sums.
-__global__ void k_adamw(float *P, float *grad, float *m, float *v, float lr, float b1,
-                        float b2, float eps, float wd, float bc1, float bc2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= MLP_NPARAM) return;
+// Sum of the blocks' partial sums of parameter i (i == MLP_NPARAM: the
+// loss), the same for every run: RED_SLICES threads each add every
+// RED_SLICES-th block's, all loads independent, then a shared-memory sum.
+// Result valid in slice 0.  Blocks adding with atomics instead (128 on each
+// address) held the gradient kernel for about 8 us after its last tile.
+constexpr int RED_PARAMS = 32, RED_SLICES = 8;
+__device__ __forceinline__ float reduce_part(const float *__restrict__ part, int nblk, int i,
+                                             float (&red)[RED_SLICES][RED_PARAMS]) {
+    const int p = threadIdx.x % RED_PARAMS, sl = threadIdx.x / RED_PARAMS;
+    float s = 0.f;
+    if (i <= MLP_NPARAM) {
+#pragma unroll 16
+        for (int b = sl; b < nblk; b += RED_SLICES) s += part[(size_t)b * TR_PART + i];
+    }
+    red[sl][p] = s;
+    __syncthreads();
+    float t = 0.f;
+    if (sl == 0)
+#pragma unroll
+        for (int k = 0; k < RED_SLICES; k++) t += red[k][p];
+    return t;
+}
+
+__global__ void __launch_bounds__(RED_PARAMS * RED_SLICES)
+k_grad_reduce(const float *__restrict__ part, int nblk, float *grad, float *loss) {
+    __shared__ float red[RED_SLICES][RED_PARAMS];
+    const int i = blockIdx.x * RED_PARAMS + threadIdx.x % RED_PARAMS;
+    const float g = reduce_part(part, nblk, i, red);
+    if (threadIdx.x >= RED_PARAMS) return;
+    if (i < MLP_NPARAM) grad[i] = g;
+    else if (i == MLP_NPARAM) *loss = g;
+}
+
+// AdamW (decoupled weight decay on the weight matrices, not the biases) on
+// the sum of the blocks' gradients; adds the batch's loss to *loss.
+__global__ void __launch_bounds__(RED_PARAMS * RED_SLICES)
+k_adamw(float *P, const float *__restrict__ part, int nblk, float *m, float *v, float *loss, float lr, float b1,
+        float b2, float eps, float wd, float bc1, float bc2) {
+    __shared__ float red[RED_SLICES][RED_PARAMS];
+    const int i = blockIdx.x * RED_PARAMS + threadIdx.x % RED_PARAMS;
+    const float g = reduce_part(part, nblk, i, red);
+    if (threadIdx.x >= RED_PARAMS || i > MLP_NPARAM) return;
+    if (i == MLP_NPARAM) { *loss += g; return; }
     const bool bias = (i >= OFF_B1 && i < OFF_W2) || (i >= OFF_B2 && i < OFF_W3) || i >= OFF_B3;
-    const float g = grad[i];
-    grad[i] = 0.f;
     const float mi = b1 * m[i] + (1.f - b1) * g;
     const float vi = b2 * v[i] + (1.f - b2) * g * g;
     m[i] = mi;
@@ -534,26 +582,41 @@ cudaError_t launch_mlp_rows(cudaStream_t s, const float *P, const float *norm, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_grad(cudaStream_t s, const float *P, const float *norm, const float *X, const float *Y,
-                            const uint32_t *idx, int bsz, float *grad, float *loss) {
+// The partial sums of a batch: nblk blocks' into part (TR_BLOCKS x TR_PART).
+static cudaError_t launch_grad_part(cudaStream_t s, const float *P, const float *norm, const float *X,
+                                    const float *Y, const uint32_t *idx, int bsz, float *part, int &nblk) {
     static size_t attr_done[MAX_DEVICES] = {};
     const size_t smem = sizeof(TrShared);
     cudaError_t e = allow_dyn_smem((const void *)k_mlp_grad, smem, attr_done);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    // two resident blocks per SM; larger batches loop over their tiles
-    const int grid = std::min((bsz + TR_S - 1) / TR_S, 2 * sms);
-    k_mlp_grad<<<grid, TR_THREADS, smem, s>>>(P, norm, X, Y, idx, bsz, grad, loss);
+    nblk = std::min((bsz + TR_S - 1) / TR_S, TR_BLOCKS);
+    k_mlp_grad<<<nblk, TR_THREADS, smem, s>>>(P, norm, X, Y, idx, bsz, part);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adamw(cudaStream_t s, float *P, float *grad, float *m, float *v, float lr, float wd,
-                         int step) {
+constexpr int RED_GRID = (MLP_NPARAM + 1 + RED_PARAMS - 1) / RED_PARAMS;
+
+// Gradient and loss of a batch (idx NULL: rows 0..bsz-1).
+cudaError_t launch_mlp_grad(cudaStream_t s, const float *P, const float *norm, const float *X, const float *Y,
+                            const uint32_t *idx, int bsz, float *part, float *grad, float *loss) {
+    int nblk = 0;
+    cudaError_t e = launch_grad_part(s, P, norm, X, Y, idx, bsz, part, nblk);
+    if (e != cudaSuccess) return e;
+    k_grad_reduce<<<RED_GRID, RED_PARAMS * RED_SLICES, 0, s>>>(part, nblk, grad, loss);
+    return cudaGetLastError();
+}
+
+// One training batch: its gradient and the AdamW update; *loss grows by the
+// batch's loss.
+cudaError_t launch_mlp_batch(cudaStream_t s, float *P, const float *norm, const float *X, const float *Y,
+                             const uint32_t *idx, int bsz, float *part, float *m, float *v, float *loss, float lr,
+                             float wd, int step) {
+    int nblk = 0;
+    cudaError_t e = launch_grad_part(s, P, norm, X, Y, idx, bsz, part, nblk);
+    if (e != cudaSuccess) return e;
     const float b1 = 0.9f, b2 = 0.999f;
     const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
-    k_adamw<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(P, grad, m, v, lr, b1, b2, 1e-8f, wd, bc1, bc2);
+    k_adamw<<<RED_GRID, RED_PARAMS * RED_SLICES, 0, s>>>(P, part, nblk, m, v, loss, lr, b1, b2, 1e-8f, wd, bc1, bc2);
     return cudaGetLastError();
 }
 
