@@ -84,14 +84,28 @@ def fp32_peak_tflops(local_rank: int = 0) -> float:
     return fp32_peak(local_rank)["tflops"]
 
 
-def kernels_per_step(ncrit, group_pack=0):
-    """reset, kick+drift+bbox, domains, keys, 8 sort passes, reorder, 4 build
+def merge_launches(n):
+    """Merge launches of the sort after its tile sort for n bodies of one
+    system (4608-key tiles, runs doubled by each launch), or None where the
+    radix sort runs (above 2^22 bodies)."""
+    return None if n > 1 << 22 else max(0, math.ceil(math.log2(n / 4608)))
+
+
+def kernels_per_step(ncrit, group_pack=0, n=None):
+    """With n, the launches of a step of n bodies: up to 2^22 the keys come
+    with the tile sort, merges follow and the last one reorders.  Else:
+    reset, kick+drift+bbox, domains, keys, 8 sort passes, reorder, 4 build
     (+2 for sibling packing of the groups), multipoles in two passes (leaves,
     then internal cells; they also write the MAC records), walk (a second
     instantiation when groups may exceed 16 bodies: three bodies per lane for
     17..24, two for more than 32), kick.  (The start-list reset before the
     multipoles is a memset node, not a kernel.)"""
-    return 21 + (1 if ncrit > 16 else 0) + (2 if group_pack else 0)
+    order = 11                                # domains, keys, 8 radix passes, reorder
+    if n is not None and merge_launches(n) is not None:
+        order = 1 + merge_launches(n)
+    return 10 + order + (1 if ncrit > 16 else 0) + (2 if group_pack else 0)
+
+
 # DRAM bytes (read + write) of one step's walk (both instantiations) from
 # the ncu capture in profiles/k_walk_plummer_n2e20.md, keyed by (N, ncrit,
 # group_pack); other choices have no capture and report null.
@@ -541,6 +555,14 @@ STAGE_BYTES = {
 
 
 def stage_bytes(n, ncells, ngroups):
+    m = merge_launches(n)
+    if m is not None:              # tiles read positions and write pairs; merges move pairs, the last one bodies
+        return {**stage_bytes_radix(n, ncells, ngroups), "keys": 28 * n if m else 88 * n,
+                "sort": 24 * n * (m - 1) + 92 * n if m else 0, "reorder": 0}
+    return stage_bytes_radix(n, ncells, ngroups)
+
+
+def stage_bytes_radix(n, ncells, ngroups):
     return {"kick_drift_domain": 88 * n, "keys": 24 * n, "sort": (20 + 7 * 24) * n,
             "reorder": 76 * n, "build": 8 * n + 16 * ncells + 8 * ngroups,
             "multipoles": 16 * n + 64 * ncells, "kick": 48 * n}
@@ -960,7 +982,7 @@ def run_ours(a, rank, world, local_rank):
                          "flops_basis": f"{FLOP_PC} per body-cell + {FLOP_PP} per body-body interaction"},
             "cpu_baseline": cpu,
             "e2e": e2e,
-            "gpu_launches": kernels_per_step(a.ncrit, a.group_pack) * a.steps,
+            "gpu_launches": kernels_per_step(a.ncrit, a.group_pack, a.n) * a.steps,
             "clocks": clocks,
             "stages_ms_per_step": {s: float(v) / a.steps for s, v in zip(B.STAGES, stages)},
             "stages_from": "as many further steps with stage events in the step graph (ms_per_step is timed without them)",

@@ -104,7 +104,7 @@ int bonsai_set_systems(bonsai_ctx *ctx, const long long *offsets, int nsys);
 
 /* Sect. 2 "sorting", "moving", "tree-construction": domain cube, 63-bit
  * Morton keys (21 bits per axis, x in the lowest bit of each triple), stable
- * LSD radix sort, body reorder, octree (cells with more than nleaf bodies
+ * sort, body reorder, octree (cells with more than nleaf bodies
  * split into their non-empty octants; breadth-first, key order within a
  * level) and walk groups (cells with at most ncrit bodies whose parent has
  * more). */
@@ -237,7 +237,9 @@ int bonsai_set_stage_timing(bonsai_ctx *ctx, int on);
 
 /* Device time of each stage of the last bonsai_step in milliseconds (that
  * step must have run with stage timing on: BONSAI_ERR_NOT_READY otherwise).
- * ms[0] first kick + drift + domain, [1] keys, [2] sort, [3] reorder, [4]
+ * ms[0] first kick + drift + domain, [1] keys, [2] sort, [3] reorder (up to
+ * 2^22 bodies of one system the sort is a merge sort: [1] then holds the keys
+ * and the sort of tiles, [2] the merges, the last of which reorders), [4]
  * tree build, [5] multipoles (with the walk's MAC records), [6] walk, [7]
  * second kick.  Synchronises; writes min(n, 8) values and returns that
  * count (negative on error). */
@@ -285,16 +287,15 @@ int bonsai_get_counts(bonsai_ctx *ctx, uint32_t *n_pc, uint32_t *n_pp,
  * allocator would fail or fragment it).  keys (n, read only), sorted_keys
  * (n) and perm (n) are caller-owned DEVICE buffers on the current device;
  * sorted_keys[i] = keys[perm[i]], equal keys in input order.  All scratch is
- * one static device array (about 0.9 MiB, held by every GPU that loads the
+ * one static device array (0.75 MiB, held by every GPU that loads the
  * library until exit), so n is limited to 65536 (larger n: INVALID_ARG).
  * The first call on a device looks up that array's device address and sets
- * the sort kernel's shared-memory limit for that device.  Every call reuses
+ * the merge kernel's shared-memory limit for that device.  Every call reuses
  * the same scratch: calls whose GPU work could overlap (other threads or
  * streams) race and must be serialised by the caller.  Work is ordered on
- * cuda_stream (NULL: the legacy default stream); the call then reads a status
- * word back and synchronises that stream, so it cannot run while the stream
- * is being captured into a CUDA graph.  It returns BONSAI_ERR_TIMEOUT if a
- * bounded device-side wait gave up.  Error text: bonsai_last_error(NULL). */
+ * cuda_stream (NULL: the legacy default stream); the call then
+ * synchronises that stream, so it cannot run while the stream is being
+ * captured into a CUDA graph.  Error text: bonsai_last_error(NULL). */
 int bonsai_sort_keys_static(const uint64_t *keys, uint64_t *sorted_keys,
                             uint32_t *perm, long long n, void *cuda_stream);
 
@@ -310,7 +311,8 @@ int bonsai_sort_keys_static(const uint64_t *keys, uint64_t *sorted_keys,
  * 1 <= blocks <= 65535, 32 <= threads <= 1024 (a multiple of 32), iters >= 1. */
 int bonsai_bench_fma(int blocks, int threads, long long iters, float *ms, double *flop);
 
-/* Testing aid for the bounded device-side waits: while tile >= 0, sort tile
+/* Testing aid for the bounded device-side waits: while tile >= 0, the
+ * context sorts with the radix sort whatever its size, and sort tile
  * `tile` (4096 keys) of every radix-sort pass of this context publishes no
  * count, so the look-back of the tile after it polls max_spin times, gives
  * up and sets the device's timeout status: bonsai_sync then returns

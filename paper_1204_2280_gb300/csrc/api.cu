@@ -371,7 +371,8 @@ int bonsai_build(bonsai_ctx *ctx) {
     Ctx &c = ctx->c;
     if (!c.have_bodies) return fail(ctx, BONSAI_ERR_NOT_READY, "bonsai_build: no bodies");
     const bool again = c.built;
-    const long long key[] = {c.n, c.arena_gen, c.nsys, c.nleaf, c.ncrit, c.group_pack, c.max_spin, again};
+    const long long key[] = {c.n, c.arena_gen, c.nsys, c.nleaf, c.ncrit, c.group_pack, c.max_spin, again,
+                             c.hold_tile};
     CK(run_cached(c, c.build_graph, key, (int)(sizeof key / sizeof key[0]), [&]() -> cudaError_t {
         cudaError_t e;
         if (again) {
@@ -769,6 +770,9 @@ int bonsai_debug_hold_sort_tile(bonsai_ctx *ctx, int tile) {
     Ctx &c = ctx->c;
     if (tile < -1) return fail(ctx, BONSAI_ERR_INVALID_ARG, "bonsai_debug_hold_sort_tile: need tile >= -1");
     const unsigned v = (unsigned)(tile + 1);
+    c.hold_tile = tile >= 0;                    // chooses the sort: nothing captured before holds
+    if (c.step_graph) { cudaGraphExecDestroy(c.step_graph); c.step_graph = nullptr; }
+    c.graph_n = -1;
     CK(cudaMemcpyAsync(&c.st->hold_tile, &v, sizeof(unsigned), cudaMemcpyHostToDevice, c.stream));
     CK(cudaStreamSynchronize(c.stream));
     return BONSAI_OK;

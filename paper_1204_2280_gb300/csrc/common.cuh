@@ -126,6 +126,7 @@ struct Ctx {
     long long n = 0, ncap = 0, ccap = 0;
     long long cells_hint = 0;         // cell count of the last tree the host read (0: none); sizes launches
     int ntiles = 0, nbblocks = 0;     // sort tiles, build blocks
+    bool hold_tile = false;           // testing aid on: the radix sort, whose tiles wait on one another
     int nsys = 1;                     // independent systems (contiguous body segments)
 
     // body arrays
@@ -274,6 +275,11 @@ cudaError_t launch_bbox(Ctx &c);
 cudaError_t launch_kick_drift_bbox(Ctx &c, float dt);
 cudaError_t launch_drift_bbox(Ctx &c, float dt);
 cudaError_t launch_keys(Ctx &c);
+bool sort_by_merge(const Ctx &c);
+cudaError_t launch_tile_sort(Ctx &c);
+cudaError_t launch_merges(Ctx &c);
+cudaError_t sort_pairs_small(const unsigned long long *keys, unsigned long long *out, unsigned long long *tmp,
+                             uint32_t *vout, uint32_t *vtmp, int n, cudaStream_t s);
 cudaError_t launch_sort(Ctx &c);
 cudaError_t launch_reorder(Ctx &c);
 cudaError_t launch_build(Ctx &c);

@@ -2,15 +2,8 @@
 //
 // Paper Sect. 2, "Sorting of the particles along a Space Filling Curve
 // (Morton)": every body gets a 63-bit Z-order key from its position quantised
-// on a 2^21 grid per axis over the domain cube.  The cube corner is the
-// per-axis minimum and its side S the smallest power of two strictly greater
-// than the largest extent, so that every quantisation below is exact:
-//   q_d = floor((x_d - mn_d) * 2^21 / S)
-// is computed as (int)(__fsub_rd(x_d, mn_d) * (2^21 / S)): the round-down
-// subtraction never exceeds the exact difference and floor(v 2^21/S)*S/2^21
-// is itself a float <= v, so both floors agree; the multiply by a power of
-// two is exact.
-#include "common.cuh"
+// on a 2^21 grid per axis over the domain cube (morton.cuh).
+#include "morton.cuh"
 
 namespace bonsai {
 
@@ -279,42 +272,15 @@ cudaError_t launch_kick_drift_bbox(Ctx &c, float dt) {
 }
 
 // ---------------------------------------------------------------------------
-// Smallest power of two strictly greater than the exact difference hi - lo.
-__device__ float pow2_above_diff(float hi, float lo) {
-    float e_rd = __fsub_rd(hi, lo), e_ru = __fsub_ru(hi, lo);
-    if (!(e_ru > 0.f)) return 0.f;
-    int ex;
-    float m = frexpf(e_ru, &ex);           // e_ru = m 2^ex, m in [0.5, 1)
-    if (e_rd == e_ru) return ldexpf(1.f, ex);          // exact: 2^(floor(log2 e) + 1)
-    return (m == 0.5f) ? e_ru : ldexpf(1.f, ex);       // inexact: smallest pow2 >= e_ru
-}
-
-// Spread the low 21 bits of v to every third bit (bit b -> bit 3b).
-__device__ __forceinline__ unsigned long long spread3(unsigned v) {
-    unsigned long long x = v & 0x1fffffu;
-    x = (x | (x << 32)) & 0x001f00000000ffffull;
-    x = (x | (x << 16)) & 0x001f0000ff0000ffull;
-    x = (x | (x << 8)) & 0x100f00f00f00f00full;
-    x = (x | (x << 4)) & 0x10c30c30c30c30c3ull;
-    x = (x | (x << 2)) & 0x1249249249249249ull;
-    return x;
-}
-
 // Domain of every system from its bounding box, and the histogram of the
 // extra radix pass on the system id (the system sizes).
 __global__ void k_domains(DevState *st, int nsys) {
     for (int sys = threadIdx.x; sys < MAX_SYSTEMS; sys += blockDim.x) {
         if (sys < nsys) {
-            float S = 0x1p-64f;
-            for (int d = 0; d < 3; d++) {
-                float lo = ord2f(st->dom[6 * sys + d]), hi = ord2f(st->dom[6 * sys + 3 + d]);
-                st->mn[3 * sys + d] = lo;
-                S = fmaxf(S, pow2_above_diff(hi, lo));
-            }
-            int ex;
-            frexpf(S, &ex);                // S = 2^(ex-1)
-            st->side[sys] = S;
-            st->scale[sys] = ldexpf(1.f, KEY_BITS_PER_AXIS - (ex - 1));
+            float mn[3], side;
+            st->scale[sys] = domain_of(st->dom + 6 * sys, mn, side);
+            st->side[sys] = side;
+            for (int d = 0; d < 3; d++) st->mn[3 * sys + d] = mn[d];
             st->hist[SORT_PASSES * SORT_RADIX + sys] = st->sys_off[sys + 1] - st->sys_off[sys];
         } else {
             st->hist[SORT_PASSES * SORT_RADIX + sys] = 0u;
@@ -347,7 +313,6 @@ k_keys(const float4 *__restrict__ p, const uint8_t *__restrict__ sysid, int n, i
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nstatus; i += gridDim.x * blockDim.x)
         status0[i] = 0;
     __syncthreads();
-    const unsigned qmax = (1u << KEY_BITS_PER_AXIS) - 1u;
     // chunks of KEYS_THREADS * KEYS_ITEMS bodies, grid-stride: a block sums
     // its chunks in shared memory and adds each digit count to the global
     // histograms once
@@ -367,12 +332,7 @@ k_keys(const float4 *__restrict__ p, const uint8_t *__restrict__ sysid, int n, i
     for (int k = 0; k < KEYS_ITEMS; k++) {
         int i = base + k * KEYS_THREADS;
         if (i < n) {
-            const float4 q = qs[k];
-            const float4 dm = s_dom[ss[k]];
-            unsigned qx = min((unsigned)(__fsub_rd(q.x, dm.x) * dm.w), qmax);
-            unsigned qy = min((unsigned)(__fsub_rd(q.y, dm.y) * dm.w), qmax);
-            unsigned qz = min((unsigned)(__fsub_rd(q.z, dm.z) * dm.w), qmax);
-            unsigned long long key = spread3(qx) | (spread3(qy) << 1) | (spread3(qz) << 2);
+            const unsigned long long key = morton_key(qs[k], s_dom[ss[k]]);
             keys[i] = key;
             // one shared-memory atomic per digit (counting the digits a warp
             // shares with one atomic per warp measured slower: 23.7 against
@@ -391,6 +351,7 @@ k_keys(const float4 *__restrict__ p, const uint8_t *__restrict__ sysid, int n, i
 cudaError_t launch_keys(Ctx &c) {
     int n = (int)c.n;
     int per = KEYS_THREADS * KEYS_ITEMS;
+    if (sort_by_merge(c)) return launch_tile_sort(c);
     cudaError_t e = launch_domains(c);
     if (e != cudaSuccess) return e;
     // The sort ping-pongs between c.keys and c.keys_alt and must end in

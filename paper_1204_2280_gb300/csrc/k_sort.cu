@@ -239,13 +239,13 @@ k_onesweep(const unsigned long long *__restrict__ kin, const uint32_t *__restric
 }
 
 constexpr size_t SORT_DYN_SMEM = (size_t)SORT_TILE * (sizeof(unsigned long long) + sizeof(uint32_t));
-extern const size_t SORT_DYN_SMEM_BYTES = SORT_DYN_SMEM;
 
 // SORT_PASSES passes over the key digits; with several systems one more
 // stable pass on the system id groups the bodies by system (key order inside
 // each).  Buffers alternate so that the result always lands in c.keys /
 // c.vals (the key kernel writes to c.keys_alt for an odd number of passes).
 cudaError_t launch_sort(Ctx &c) {
+    if (sort_by_merge(c)) return launch_merges(c);
     static size_t attr_done[MAX_DEVICES] = {};
     cudaError_t ea = allow_dyn_smem((const void *)k_onesweep, SORT_DYN_SMEM, attr_done);
     if (ea != cudaSuccess) return ea;

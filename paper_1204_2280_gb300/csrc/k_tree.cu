@@ -33,6 +33,7 @@ __global__ void k_reorder(const uint32_t *__restrict__ perm, const float4 *__res
 }
 
 cudaError_t launch_reorder(Ctx &c) {
+    if (sort_by_merge(c)) return cudaSuccess;     // the last merge moved the bodies
     int n = (int)c.n;
     k_reorder<<<(n + 255) / 256, 256, 0, c.stream>>>(c.vals, c.pos4_alt, c.vel4_alt, c.id_alt, n,
                                                      c.pos4, c.vel4, c.id);

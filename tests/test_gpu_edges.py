@@ -44,3 +44,50 @@ def test_normalisation_blocks(n):
         x, y = X.astype(np.float64), Y.astype(np.float64)
         ref = np.concatenate([x.mean(0), np.maximum(x.std(0), 1e-6), [np.sqrt((y * y).mean())]])
         assert np.abs(norm - ref).max() <= 1e-6 * np.abs(ref).max()
+
+
+def _stable(keys):
+    return np.argsort(keys, kind="stable")
+
+
+@pytest.mark.parametrize("n", [1, 2, 4607, 4608, 4609, 9216, 9217, 13825, 65536])
+def test_merge_sort_tiles(n):
+    """The static sort at the edges of its 4608-key tiles and runs, with few
+    distinct keys (long runs of equal ones), reversed keys and random ones:
+    equal to numpy's stable sort."""
+    import torch
+    rng = np.random.default_rng(n)
+    for keys in (rng.integers(0, 3, n), np.arange(n)[::-1].copy(), rng.integers(0, 2 ** 62, n) * 2 + 1,
+                 np.full(n, 2 ** 63 - 1)):
+        k = torch.from_numpy(keys.astype(np.int64)).cuda()
+        out, perm = torch.empty_like(k), torch.empty(n, dtype=torch.int32, device="cuda")
+        B.bonsai_sort_keys_static(k, out, perm)
+        ref = _stable(keys)
+        assert np.array_equal(perm.cpu().numpy(), ref)
+        assert np.array_equal(out.cpu().numpy(), keys[ref])
+
+
+@pytest.mark.parametrize("n", [1, 4608, 4609, 9217, 36865, (1 << 20) - 1, 1 << 20, (1 << 20) + 1])
+def test_build_order_across_sorts(n):
+    """Keys, permutation and moved bodies of a build on both sides of the
+    tile, run and sort choices, with duplicate positions, against the
+    oracle's keys and a stable sort; a rebuild from the sorted state keeps
+    the order."""
+    import oracle
+    rng = np.random.default_rng(n)
+    pos = rng.normal(size=(n, 3)).astype(np.float32)
+    pos[n // 2:n // 2 + n // 8] = pos[0]
+    mass = rng.uniform(0.5, 1.5, n).astype(np.float32)
+    mn, S = oracle.domain(pos)
+    k = oracle.keys(pos, mn, S)
+    ref = _stable(k)
+    with B.Bonsai(B.Config(ncrit=32)) as bz:
+        bz.set_bodies(pos, mass, pos)
+        for _ in range(2):
+            bz.build()
+            kk, pp = B.bonsai_get_keys(bz.ctx)
+            assert np.array_equal(kk, k[ref]) and np.array_equal(pp, ref)
+            x, v = np.zeros((n, 3), np.float32), np.zeros((n, 3), np.float32)
+            B.bonsai_get_bodies(bz.ctx, x, v)
+            assert np.array_equal(x, pos) and np.array_equal(v, pos)
+        bz.sync()
