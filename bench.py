@@ -96,7 +96,7 @@ def kernels_per_step(ncrit, group_pack=0, n=None):
     with the tile sort, merges follow and the last one reorders.  Else:
     reset, kick+drift+bbox, domains, keys, 8 sort passes, reorder, 4 build
     (+2 for sibling packing of the groups), multipoles in two passes (leaves,
-    then internal cells; they also write the MAC records), walk (a second
+    then internal cells), walk (a second
     instantiation when groups may exceed 16 bodies: three bodies per lane for
     17..24, two for more than 32), kick.  (The start-list reset before the
     multipoles is a memset node, not a kernel.)"""
@@ -549,7 +549,7 @@ STAGE_BYTES = {
     "sort": "8 passes: pass 0 reads keys (8 B), later passes keys + values (12 B); each writes 12 B",
     "reorder": "perm, pos, vel, id read (40 B); pos, vel, id written (36 B)",
     "build": "sorted keys read (8 B/body); 16 B per cell and 8 B per group written",
-    "multipoles": "pos read (16 B/body); 64 B per cell written (com, M, Q, delta, MAC record)",
+    "multipoles": "pos read (16 B/body); 48 B per cell written (com, M, Q, delta)",
     "kick": "vel, acc read (32 B); vel written (16 B)",
 }
 
@@ -565,7 +565,7 @@ def stage_bytes(n, ncells, ngroups):
 def stage_bytes_radix(n, ncells, ngroups):
     return {"kick_drift_domain": 88 * n, "keys": 24 * n, "sort": (20 + 7 * 24) * n,
             "reorder": 76 * n, "build": 8 * n + 16 * ncells + 8 * ngroups,
-            "multipoles": 16 * n + 64 * ncells, "kick": 48 * n}
+            "multipoles": 16 * n + 48 * ncells, "kick": 48 * n}
 
 
 def run_sph(a, dev, stream):

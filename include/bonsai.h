@@ -240,7 +240,7 @@ int bonsai_set_stage_timing(bonsai_ctx *ctx, int on);
  * ms[0] first kick + drift + domain, [1] keys, [2] sort, [3] reorder (up to
  * 2^22 bodies of one system the sort is a merge sort: [1] then holds the keys
  * and the sort of tiles, [2] the merges, the last of which reorders), [4]
- * tree build, [5] multipoles (with the walk's MAC records), [6] walk, [7]
+ * tree build, [5] multipoles, [6] walk, [7]
  * second kick.  Synchronises; writes min(n, 8) values and returns that
  * count (negative on error). */
 int bonsai_get_stage_times(bonsai_ctx *ctx, float *ms, int n);

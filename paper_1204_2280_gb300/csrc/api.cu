@@ -82,7 +82,7 @@ cudaError_t alloc_bodies(Ctx &c, long long n) {
     a.take(c.cell_level, ccap, plan); a.take(c.cell_parent, ccap, plan);
     a.take(c.cell_done, ccap, plan); a.take(c.cell_cb, ccap, plan); a.take(c.cell_start, ccap, plan);
     a.take(c.mono, ccap, plan); a.take(c.quadA, ccap, plan); a.take(c.quadB, ccap, plan);
-    a.take(c.test, ccap, plan); a.take(c.delta, ccap, plan); a.take(c.cext, ccap, plan);
+    a.take(c.delta, ccap, plan); a.take(c.cext, ccap, plan);
     a.take(c.shadow, 10 * (size_t)(ccap < 585 * MAX_SYSTEMS ? ccap : 585 * MAX_SYSTEMS), plan);   // FP64 root terms of the level-1 cells
     a.take(c.groups, n, plan); a.take(c.groups_raw, n, plan);
     a.take(c.group_lvl, n, plan); a.take(c.group_flag, n, plan); a.take(c.group_bcount, (n + PACK_THREADS - 1) / PACK_THREADS, plan);
@@ -172,9 +172,7 @@ cudaError_t pipeline_tree(Ctx &c) {
 }
 
 cudaError_t pipeline_forces(Ctx &c, float theta, float eps) {
-    cudaError_t e;
-    if ((e = launch_open_radius(c, theta)) != cudaSuccess) return e;
-    return launch_walk(c, eps);
+    return launch_walk(c, theta, eps);
 }
 
 // One kick-drift-kick step; events between the stages give per-stage times.
@@ -194,11 +192,8 @@ cudaError_t pipeline_step(Ctx &c, float dt) {
     STAGE(2, launch_sort(c));
     STAGE(3, launch_reorder(c));
     STAGE(4, launch_build(c));
-    // Plain steps: the multipole pass also writes the MAC records for the
-    // step's theta (the learned path sets its own opening angles).
-    const bool plain = c.mlp_P == nullptr;
-    STAGE(5, launch_multipoles(c, plain ? c.theta : 0.f));
-    STAGE(6, plain ? launch_walk(c, c.eps) : pipeline_learned_forces(c, c.eps));
+    STAGE(5, launch_multipoles(c));
+    STAGE(6, c.mlp_P == nullptr ? launch_walk(c, c.theta, c.eps) : pipeline_learned_forces(c, c.eps));
     STAGE(7, launch_kick(c, dt));
 #undef STAGE
     return c.stage_timing ? cudaEventRecordWithFlags(c.ev[8], c.stream, evf) : cudaSuccess;

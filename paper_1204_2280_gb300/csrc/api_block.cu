@@ -208,10 +208,9 @@ static cudaError_t block_cycle(Ctx &c, float dt_max, int kmax, float eta, int re
             k_block_drift<<<grid, 256, 0, c.stream>>>(c.pos4, c.vel4, n, dtm, quiet + 1u);
             if ((e = launch_multipoles_refit(c)) != cudaSuccess) return e;
         }
-        if ((e = launch_open_radius(c, c.theta)) != cudaSuccess) return e;
         c.block_kmax = kmax;
         c.block_s = nx;
-        e = launch_walk(c, c.eps);
+        e = launch_walk(c, c.theta, c.eps);
         c.block_kmax = -1;
         if (e != cudaSuccess) return e;
         c.blk_walked++;

@@ -73,8 +73,7 @@ cudaError_t pipeline_learned_forces(Ctx &c, float eps) {
     const unsigned *gate = &c.st->judge_on;
     k_judge_gate<<<1, 32, 0, c.stream>>>(c.st, c.judge_every);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_open_radius(c, c.theta_coarse)) != cudaSuccess) return e;
-    if ((e = launch_walk(c, eps, true)) != cudaSuccess) return e;
+    if ((e = launch_walk(c, c.theta_coarse, eps, true)) != cudaSuccess) return e;
     if ((e = launch_mlp_infer(c, c.mlp_P, c.mlp_norm)) != cudaSuccess) return e;
     if ((e = launch_judge_targets(c)) != cudaSuccess) return e;
     if ((e = launch_direct(c, c.judge_targets, c.judge_n, eps, c.judge_partial, JUDGE_SPLIT, c.judge_direct,
@@ -83,8 +82,7 @@ cudaError_t pipeline_learned_forces(Ctx &c, float eps) {
     if ((e = launch_judge(c, c.judge_targets, c.judge_n, c.judge_direct, c.p99_budget, gate)) != cudaSuccess)
         return e;
     if ((e = launch_gated_walk_reset(c)) != cudaSuccess) return e;
-    if ((e = launch_open_radius(c, c.theta_fine, &c.st->fallback)) != cudaSuccess) return e;
-    return launch_walk(c, eps, false, &c.st->fallback);
+    return launch_walk(c, c.theta_fine, eps, false, &c.st->fallback);
 }
 
 }  // namespace bonsai
@@ -366,8 +364,7 @@ int bonsai_learn_samples(bonsai_ctx *ctx, float theta, float eps, int ntar, unsi
     c.graph_n = -1;
     CCK(cudaMemcpyAsync(tg, pool.data(), sizeof(uint32_t) * ntar, cudaMemcpyHostToDevice, c.stream));
     CCK(launch_reset(c));
-    CCK(launch_open_radius(c, theta));
-    CCK(launch_walk(c, eps, true));
+    CCK(launch_walk(c, theta, eps, true));
     CCK(launch_direct(c, tg, ntar, eps, c.judge_partial, JUDGE_SPLIT, c.judge_direct));
     float *dX = X, *dY = Y, *owned = nullptr;
     uint32_t *dI = ids;

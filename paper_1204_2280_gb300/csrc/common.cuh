@@ -8,7 +8,7 @@
 //   cells (capacity C): body uint2 (begin, count), link uint2 (internal:
 //     child_begin, nchild; leaf: begin, count | LEAF_BIT), level u8,
 //     parent u32, done u32, mono float4 (com, M), quadA float4 (-Q: xx yy zz xy),
-//     quadB float2 (-Q: xz yz), test float4 (com, r_open), delta float
+//     quadB float2 (-Q: xz yz), delta float2 (|com - centre|, side)
 //   groups (capacity N): uint2 (begin, count); with sibling packing the
 //     unpacked groups (uint2), their levels (u8) and start flags (u8) too
 #pragma once
@@ -145,7 +145,7 @@ struct Ctx {
     uint8_t *cell_level = nullptr;
     uint32_t *cell_parent = nullptr, *cell_done = nullptr, *cell_cb = nullptr;
     uint32_t *cell_start = nullptr;  // multipoles: the internal cells whose children are all leaves
-    float4 *mono = nullptr, *quadA = nullptr, *test = nullptr;
+    float4 *mono = nullptr, *quadA = nullptr;
     float2 *quadB = nullptr;
     float2 *delta = nullptr;         // per cell: (|com - centre|, side l; after a refit 2 ext)
     float4 *cext = nullptr;          // per cell after a refit: build-time centre, half side ext holding its bodies
@@ -284,12 +284,11 @@ cudaError_t launch_sort(Ctx &c);
 cudaError_t launch_reorder(Ctx &c);
 cudaError_t launch_build(Ctx &c);
 cudaError_t launch_internal_counts(Ctx &c);
-cudaError_t launch_multipoles(Ctx &c, float theta = 0.f);
+cudaError_t launch_multipoles(Ctx &c);
 cudaError_t launch_multipoles_refit(Ctx &c);
 cudaError_t launch_cell_cubes(Ctx &c);
 cudaError_t launch_sph_walk(Ctx &c, const float *hs, const float4 *cext, float *rho_s, int32_t *cnt_s);
-cudaError_t launch_open_radius(Ctx &c, float theta, const unsigned *gate = nullptr);
-cudaError_t launch_walk(Ctx &c, float eps, bool features = false, const unsigned *gate = nullptr);
+cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features = false, const unsigned *gate = nullptr);
 cudaError_t launch_direct(Ctx &c, const uint32_t *targets, int ntar, float eps, float4 *partial, int nsplit,
                           float4 *out, const unsigned *gate = nullptr);
 cudaError_t launch_judge(Ctx &c, const uint32_t *targets, int ntar, const float4 *direct, float budget,

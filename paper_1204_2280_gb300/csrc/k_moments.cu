@@ -95,15 +95,6 @@ __device__ __forceinline__ void store32(int c, const Mom32 &m, float4 *mono, flo
     qb[c] = make_float2(-m.q[4], -m.q[5]);
 }
 
-// delta[c] = (|com - centre|, side) and, when the step folds the opening
-// radius in (test != nullptr), the walk's MAC record of the cell,
-// test[c] = (com, side / theta + |com - centre|).
-__device__ __forceinline__ void put_delta(unsigned c, const Mom32 &m, float2 dl, float2 *delta, float4 *test,
-                                          float inv_theta) {
-    delta[c] = dl;
-    if (test) test[c] = make_float4(m.x, m.y, m.z, fmaf(dl.y, inv_theta, dl.x));
-}
-
 // FP64 terms of level-1 cell c for its root: with O the root cube's centre
 // (from a key inside the cell) and e = com - O, (m, m e, Q + m (3 e e^T -
 // |e|^2 I)); published by the arrival atomic on the root that follows.
@@ -159,8 +150,7 @@ struct MomArrays {
     float4 *mono, *qa;
     float2 *qb, *delta;
     double *shadow;
-    float4 *cext, *test;
-    float inv_theta;
+    float4 *cext;
     bool multi;                       // several systems (else every body is in system 0)
     uint32_t *starts;                 // internal cells whose children are all leaves
     unsigned *nstart;                 // their number
@@ -229,11 +219,10 @@ __device__ __forceinline__ void leaf_finish(unsigned c, int lev, unsigned long l
     m.q[3] = 3.f * fmaf(-sx, cy, sxy); m.q[4] = 3.f * fmaf(-sx, cz, sxz); m.q[5] = 3.f * fmaf(-sy, cz, syz);
     store32(c, m, a.mono, a.qa, a.qb);
     if (REFIT) {
-        put_delta(c, m, make_float2(com_offset(make_float3(m.x, m.y, m.z), ctr), 2.f * ext), a.delta, a.test,
-                  a.inv_theta);
+        a.delta[c] = make_float2(com_offset(make_float3(m.x, m.y, m.z), ctr), 2.f * ext);
         a.cext[c] = make_float4(ctr.x, ctr.y, ctr.z, ext);
     } else {
-        put_delta(c, m, cell_delta(kb, lev, sysb, make_float3(m.x, m.y, m.z), a.stc), a.delta, a.test, a.inv_theta);
+        a.delta[c] = cell_delta(kb, lev, sysb, make_float3(m.x, m.y, m.z), a.stc);
     }
     if (lev == 1) root_terms(c, m, kb, sysb, a.stc, a.shadow);
 }
@@ -344,11 +333,10 @@ __device__ __forceinline__ void combine_cell(unsigned c, int lv, uint2 plk, unsi
             const float4 ce = __ldcg(a.cext + cb + k);
             e = fmaxf(e, dist_inf(make_float3(ce.x, ce.y, ce.z), pc) + ce.w);
         }
-        put_delta(c, m, make_float2(com_offset(make_float3(m.x, m.y, m.z), pc), 2.f * e), a.delta, a.test,
-                  a.inv_theta);
+        a.delta[c] = make_float2(com_offset(make_float3(m.x, m.y, m.z), pc), 2.f * e);
         a.cext[c] = make_float4(pc.x, pc.y, pc.z, e);
     } else {
-        put_delta(c, m, cell_delta(kb, lv, sysb, make_float3(m.x, m.y, m.z), a.stc), a.delta, a.test, a.inv_theta);
+        a.delta[c] = cell_delta(kb, lv, sysb, make_float3(m.x, m.y, m.z), a.stc);
     }
     if (lv == 1) root_terms(c, m, kb, sysb, a.stc, a.shadow);
 }
@@ -449,10 +437,9 @@ static unsigned multipole_blocks(const Ctx &c) {
     return (unsigned)((cells + 255) / 256);
 }
 
-static MomArrays mom_arrays(Ctx &c, float theta, bool refit) {
+static MomArrays mom_arrays(Ctx &c, bool refit) {
     return MomArrays{c.st, c.cell_body, c.cell_link, c.cell_level, c.cell_parent, c.cell_done, c.pos4, c.keys,
-                     c.sysid, c.mono, c.quadA, c.quadB, c.delta, c.shadow, refit ? c.cext : nullptr,
-                     theta > 0.f ? c.test : nullptr, theta > 0.f ? 1.0f / theta : 0.f, c.nsys > 1,
+                     c.sysid, c.mono, c.quadA, c.quadB, c.delta, c.shadow, refit ? c.cext : nullptr, c.nsys > 1,
                      c.cell_start, &c.st->mom_starts};
 }
 
@@ -466,16 +453,12 @@ static cudaError_t launch_mom(Ctx &c, const MomArrays &a) {
     return cudaGetLastError();
 }
 
-// theta > 0: also the walk's MAC records for that opening angle (what
-// launch_open_radius writes), so that a step needs no separate pass.
-cudaError_t launch_multipoles(Ctx &c, float theta) {
-    return launch_mom<false>(c, mom_arrays(c, theta, false));
-}
+cudaError_t launch_multipoles(Ctx &c) { return launch_mom<false>(c, mom_arrays(c, false)); }
 
 // Moments of the existing cells at the bodies' current positions (block time
 // steps between rebuilds), with each cell's cube enlarged to hold its bodies.
 cudaError_t launch_multipoles_refit(Ctx &c) {
-    return launch_mom<true>(c, mom_arrays(c, 0.f, true));
+    return launch_mom<true>(c, mom_arrays(c, true));
 }
 
 // cext[c] = (geometric centre, l / 2) of every cell from its first body's
@@ -496,26 +479,6 @@ __global__ void k_cell_cubes(const DevState *__restrict__ st, const uint2 *__res
 cudaError_t launch_cell_cubes(Ctx &c) {
     const unsigned grid = (unsigned)min((c.ccap + 255) / 256, (long long)c.num_sms * 8);
     k_cell_cubes<<<grid, 256, 0, c.stream>>>(c.st, c.cell_body, c.cell_level, c.keys, c.sysid, c.cext);
-    return cudaGetLastError();
-}
-
-// test[c] = (com, l/theta + delta), l = S / 2^level: the opening radius of
-// the Barnes (1994) criterion as read here.
-__global__ void k_open_radius(const DevState *__restrict__ st, const float4 *__restrict__ mono,
-                              const float2 *__restrict__ delta, float inv_theta, float4 *test,
-                              const unsigned *__restrict__ gate) {
-    if (gate && *gate == 0u) return;
-    const unsigned nc = st->ncells;
-    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-        const float4 m = mono[c];
-        const float2 dl = delta[c];
-        test[c] = make_float4(m.x, m.y, m.z, fmaf(dl.y, inv_theta, dl.x));
-    }
-}
-
-cudaError_t launch_open_radius(Ctx &c, float theta, const unsigned *gate) {
-    const unsigned grid = (unsigned)min((c.ccap + 255) / 256, (long long)c.num_sms * 8);
-    k_open_radius<<<grid, 256, 0, c.stream>>>(c.st, c.mono, c.delta, 1.0f / theta, c.test, gate);
     return cudaGetLastError();
 }
 

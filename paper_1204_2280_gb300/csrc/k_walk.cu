@@ -8,11 +8,12 @@
 //  * a stack of child ranges (first child, count <= 8) in shared memory; each
 //    round pops up to 32 cells, one per lane, and tests them against the
 //    group's bounding box: a cell is opened when the squared distance from its
-//    com to the box is below r_open^2 (r_open = l/theta + delta);
+//    com to the box is below r_open^2 (r_open = l/theta + delta, formed here
+//    from the cell's l and delta);
 //  * accepted cells are staged (com, M, Q) into a 64-slot ring in shared
 //    memory; the bodies of opened leaves into a second ring; opened internal
 //    cells push their child range;
-//  * whenever a ring holds 32 sources the warp evaluates that tile: every
+//  * whenever a ring holds a tile of 32 sources the warp evaluates it: every
 //    lane streams the sources from shared memory (broadcast reads) two at a
 //    time through the packed FP32x2 instructions (add/mul/fma .f32x2, one
 //    issue slot for two operations).  Groups of <= 32 bodies: a group of n
@@ -37,6 +38,8 @@ namespace bonsai {
 
 constexpr int RING = 64;          // sources per ring
 constexpr int RPAIR = RING / 2;   // source pairs per ring
+constexpr int TILE = 32;          // sources per tile
+__device__ __forceinline__ int ring_at(int s) { return s & (RING - 1); }
 #ifndef WALK_UNROLL
 #define WALK_UNROLL 8             // unroll depth of the tile loops (4: 1% slower, 16: 9% slower)
 #endif
@@ -168,39 +171,36 @@ __device__ __forceinline__ void commit(const Part2 (&P)[BPL], Acc (&A)[BPL]) {
     }
 }
 
-// Tile evaluation.  NPH lanes share one body and split the tile's 16 source
-// pairs (lane phase p takes pairs p, p+NPH, ...): the trip count 16/NPH and
-// the stride are compile-time constants, so the shared-memory reads use
-// immediate offsets and there is no per-interaction loop bookkeeping.  Each
-// lane holds BPL bodies that reuse every source read.  Partial tiles are
-// padded with massless sources far away, which add exactly zero.
-template <int NPH, int BPL, int STRIDE>
-__device__ __forceinline__ void eval_pc(const float4 *__restrict__ base, int phase, const float4 (&me)[BPL],
-                                        const float2 eps2, Acc (&A)[BPL]) {
-    constexpr int T = 16 / NPH;
-    const int k0 = phase;
-    Me2 m[BPL];
-    Part2 P[BPL];
-#pragma unroll
-    for (int b = 0; b < BPL; b++) {
-        m[b] = me2_of(me[b]);
-        P[b] = Part2{make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    }
-#pragma unroll kWalkUnroll
-    for (int j = 0; j < T; j++) {
-        const int k = k0 + j * NPH;
-        const float4 v0 = base[k], v1 = base[STRIDE + k], v2 = base[2 * STRIDE + k],
-                     v3 = base[3 * STRIDE + k], v4 = base[4 * STRIDE + k];
+// Tile evaluation: nsrc <= 32 sources of a ring (PC: cells, else bodies) from
+// place head, a multiple of 32.  NPH lanes share one body and split the
+// source pairs (lane phase p takes pairs p, p+NPH, ...); each lane holds BPL
+// bodies that reuse every source read.  A full tile has a compile-time trip
+// count 16/NPH and stride, so the shared-memory reads use immediate offsets
+// and there is no per-interaction loop bookkeeping.  The last tile of a group
+// takes a rolled loop over the sources it has, padded to 2 NPH with massless
+// ones far away (they add exactly zero): padding it to a full tile instead
+// evaluated 16 sources too many per group and kind on average (2014 against
+// 1977 us for a step of 2^20 bodies).  Tiles of 64 sources (half the commits
+// where two or more lanes share a body) in rings of 96 were slower: 2105 us,
+// the larger rings taking the L1's room.
+template <bool PC, int BPL>
+__device__ __forceinline__ void eval_pair(const float4 *__restrict__ p, const Me2 (&m)[BPL], const float2 eps2,
+                                          Part2 (&P)[BPL]) {
+    if constexpr (PC) {
+        const float4 v0 = p[0], v1 = p[RPAIR], v2 = p[2 * RPAIR], v3 = p[3 * RPAIR], v4 = p[4 * RPAIR];
 #pragma unroll
         for (int b = 0; b < BPL; b++) pc_two(v0, v1, v2, v3, v4, m[b], eps2, P[b]);
+    } else {
+        const float4 v0 = p[0], v1 = p[RPAIR];
+#pragma unroll
+        for (int b = 0; b < BPL; b++) pp_two(v0, v1, m[b], eps2, P[b]);
     }
-    commit<BPL>(P, A);
 }
-template <int NPH, int BPL, int STRIDE>
-__device__ __forceinline__ void eval_pp(const float4 *__restrict__ base, int phase, const float4 (&me)[BPL],
-                                        const float2 eps2, Acc (&A)[BPL]) {
+
+template <bool PC, int NPH, int BPL>
+__device__ __forceinline__ void eval_tile(const float4 *__restrict__ ring, int head, int nsrc, int phase,
+                                          const float4 (&me)[BPL], const float2 eps2, Acc (&A)[BPL]) {
     constexpr int T = 16 / NPH;
-    const int k0 = phase;
     Me2 m[BPL];
     Part2 P[BPL];
 #pragma unroll
@@ -208,12 +208,13 @@ __device__ __forceinline__ void eval_pp(const float4 *__restrict__ base, int pha
         m[b] = me2_of(me[b]);
         P[b] = Part2{make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     }
+    const float4 *base = ring + (head >> 1) + phase;
+    if (nsrc == TILE) {
 #pragma unroll kWalkUnroll
-    for (int j = 0; j < T; j++) {
-        const int k = k0 + j * NPH;
-        const float4 v0 = base[k], v1 = base[STRIDE + k];
-#pragma unroll
-        for (int b = 0; b < BPL; b++) pp_two(v0, v1, m[b], eps2, P[b]);
+        for (int j = 0; j < T; j++) eval_pair<PC, BPL>(base + j * NPH, m, eps2, P);
+    } else {
+#pragma unroll 1
+        for (int k = 0; 2 * k < nsrc; k += NPH) eval_pair<PC, BPL>(base + k, m, eps2, P);
     }
     commit<BPL>(P, A);
 }
@@ -251,39 +252,21 @@ __device__ __forceinline__ int walk_lg(int ng) {
 }
 
 // Warp-uniform dispatch on log2(body slots).
-template <int BPL, int STRIDE>
-__device__ __forceinline__ void tile_pc(int lg, const float4 *__restrict__ base, int phase, const float4 (&me)[BPL],
-                                        const float2 eps2, Acc (&A)[BPL]) {
+template <bool PC, int BPL>
+__device__ __forceinline__ void tile_eval(int lg, const float4 *__restrict__ ring, int head, int nsrc, int phase,
+                                          const float4 (&me)[BPL], const float2 eps2, Acc (&A)[BPL]) {
     if constexpr (BPL == 3) {
-        eval_pc<4, 3, STRIDE>(base, phase, me, eps2, A);
+        eval_tile<PC, 4, 3>(ring, head, nsrc, phase, me, eps2, A);
     } else if constexpr (BPL == 2) {
-        if (lg == 4) eval_pc<2, 2, STRIDE>(base, phase, me, eps2, A);
-        else eval_pc<1, 2, STRIDE>(base, phase, me, eps2, A);
+        if (lg == 4) eval_tile<PC, 2, 2>(ring, head, nsrc, phase, me, eps2, A);
+        else eval_tile<PC, 1, 2>(ring, head, nsrc, phase, me, eps2, A);
     } else {
         switch (lg) {
-            case 1: eval_pc<16, 1, STRIDE>(base, phase, me, eps2, A); break;
-            case 2: eval_pc<8, 1, STRIDE>(base, phase, me, eps2, A); break;
-            case 3: eval_pc<4, 1, STRIDE>(base, phase, me, eps2, A); break;
-            case 4: eval_pc<2, 1, STRIDE>(base, phase, me, eps2, A); break;
-            default: eval_pc<1, 1, STRIDE>(base, phase, me, eps2, A); break;
-        }
-    }
-}
-template <int BPL, int STRIDE>
-__device__ __forceinline__ void tile_pp(int lg, const float4 *__restrict__ base, int phase, const float4 (&me)[BPL],
-                                        const float2 eps2, Acc (&A)[BPL]) {
-    if constexpr (BPL == 3) {
-        eval_pp<4, 3, STRIDE>(base, phase, me, eps2, A);
-    } else if constexpr (BPL == 2) {
-        if (lg == 4) eval_pp<2, 2, STRIDE>(base, phase, me, eps2, A);
-        else eval_pp<1, 2, STRIDE>(base, phase, me, eps2, A);
-    } else {
-        switch (lg) {
-            case 1: eval_pp<16, 1, STRIDE>(base, phase, me, eps2, A); break;
-            case 2: eval_pp<8, 1, STRIDE>(base, phase, me, eps2, A); break;
-            case 3: eval_pp<4, 1, STRIDE>(base, phase, me, eps2, A); break;
-            case 4: eval_pp<2, 1, STRIDE>(base, phase, me, eps2, A); break;
-            default: eval_pp<1, 1, STRIDE>(base, phase, me, eps2, A); break;
+            case 1: eval_tile<PC, 16, 1>(ring, head, nsrc, phase, me, eps2, A); break;
+            case 2: eval_tile<PC, 8, 1>(ring, head, nsrc, phase, me, eps2, A); break;
+            case 3: eval_tile<PC, 4, 1>(ring, head, nsrc, phase, me, eps2, A); break;
+            case 4: eval_tile<PC, 2, 1>(ring, head, nsrc, phase, me, eps2, A); break;
+            default: eval_tile<PC, 1, 1>(ring, head, nsrc, phase, me, eps2, A); break;
         }
     }
 }
@@ -336,9 +319,6 @@ __device__ __forceinline__ void walk_pop(const unsigned *stk, int &sp, int lane,
 #ifndef WALK_MIN_BLOCKS2
 #define WALK_MIN_BLOCKS2 0
 #endif
-#ifndef WALK_SPEC_LOADS
-#define WALK_SPEC_LOADS 1           // 1: load a tested cell's moments with its MAC record
-#endif
 #ifndef WALK_SMALL_LAST
 #define WALK_SMALL_LAST 16          // > 0: groups of at most this many bodies in a second pass
 #endif
@@ -353,7 +333,7 @@ __device__ __forceinline__ void walk_pop(const unsigned *stk, int &sp, int lane,
 template <int BPL, bool FEAT, bool BLOCK>
 __global__ void WALK_ATTRS
 k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__ groups,
-       const float4 *__restrict__ pos4, const float4 *__restrict__ test,
+       const float4 *__restrict__ pos4, const float2 *__restrict__ delta, float inv_theta,
        const uint2 *__restrict__ link, const float4 *__restrict__ mono,
        const float4 *__restrict__ quadA, const float2 *__restrict__ quadB,
        const uint8_t *__restrict__ sysid, float eps, int stack_cap, unsigned max_rounds,
@@ -479,34 +459,30 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
 
             bool open = false, acc = false, isleaf = false;
             uint2 lk = make_uint2(0u, 0u);
-#if WALK_SPEC_LOADS
             float4 cmo = make_float4(0.f, 0.f, 0.f, 0.f), cqa = cmo;
             float2 cqb = make_float2(0.f, 0.f);
-#endif
             if (has) {
-                const float4 tc = __ldg(test + cell);
+                // everything of the cell, in case it is accepted: one round
+                // trip per round.  The opening radius l/theta + |com - centre|
+                // comes from the cell's (|com - centre|, l): 56 bytes a cell.
+                cmo = __ldg(mono + cell);
+                const float2 dl = __ldg(delta + cell);
                 lk = __ldg(link + cell);
-#if WALK_SPEC_LOADS
-                // the moments, in case the cell is accepted: one round trip per round
-                cmo = __ldg(mono + cell); cqa = __ldg(quadA + cell); cqb = __ldg(quadB + cell);
-#endif
-                const float dx = fmaxf(fmaxf(bx0 - tc.x, tc.x - bx1), 0.f);
-                const float dy = fmaxf(fmaxf(by0 - tc.y, tc.y - by1), 0.f);
-                const float dz = fmaxf(fmaxf(bz0 - tc.z, tc.z - bz1), 0.f);
+                cqa = __ldg(quadA + cell); cqb = __ldg(quadB + cell);
+                const float dx = fmaxf(fmaxf(bx0 - cmo.x, cmo.x - bx1), 0.f);
+                const float dy = fmaxf(fmaxf(by0 - cmo.y, cmo.y - by1), 0.f);
+                const float dz = fmaxf(fmaxf(bz0 - cmo.z, cmo.z - bz1), 0.f);
                 const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                open = d2 < tc.w * tc.w;
+                const float ro = fmaf(dl.y, inv_theta, dl.x);
+                open = d2 < ro * ro;
                 acc = !open;
                 isleaf = (lk.y & LEAF_BIT) != 0u;
             }
             // Accepted cells -> body-cell ring.
             const unsigned am = __ballot_sync(0xffffffffu, acc);
             if (acc) {
-                const int s = (pc_head + pc_n + __popc(am & lt)) & (RING - 1);
-#if WALK_SPEC_LOADS
+                const int s = ring_at(pc_head + pc_n + __popc(am & lt));
                 put_cell(R, s, cmo, cqa, cqb);
-#else
-                put_cell(R, s, __ldg(mono + cell), __ldg(quadA + cell), __ldg(quadB + cell));
-#endif
             }
             pc_n += __popc(am);
             npc += __popc(am);
@@ -553,40 +529,37 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
                     const uint2 li = R.leaf[before + __popc(starts & upto) - 1];
                     const int nb = (int)min(32u, total - base);
                     if (lane < nb)
-                        put_body(R, (pp_head + pp_n + lane) & (RING - 1), __ldg(pos4 + li.x + (base + lane - li.y)));
+                        put_body(R, ring_at(pp_head + pp_n + lane), __ldg(pos4 + li.x + (base + lane - li.y)));
                     pp_n += nb;
-                    if (pp_n >= 32) {
+                    if (pp_n >= TILE) {
                         __syncwarp();
-                        tile_pp<BPL, RPAIR>(lg, R.b0 + (pp_head >> 1), phase, me, eps2x2, A);
+                        tile_eval<false, BPL>(lg, R.b0, pp_head, TILE, phase, me, eps2x2, A);
                         __syncwarp();
-                        pp_head = (pp_head + 32) & (RING - 1);
-                        pp_n -= 32;
+                        pp_head = ring_at(pp_head + TILE);
+                        pp_n -= TILE;
                     }
                 }
             }
             __syncwarp();
-            if (pc_n >= 32) {
-                tile_pc<BPL, RPAIR>(lg, R.c0 + (pc_head >> 1), phase, me, eps2x2, A);
-                pc_head = (pc_head + 32) & (RING - 1);
-                pc_n -= 32;
+            if (pc_n >= TILE) {
+                tile_eval<true, BPL>(lg, R.c0, pc_head, TILE, phase, me, eps2x2, A);
+                pc_head = ring_at(pc_head + TILE);
+                pc_n -= TILE;
             }
             __syncwarp();
         }
-        // Remaining partial tiles (head is 0 or 32, n < 32): pad to 32 with
-        // massless sources far away, then evaluate as full tiles.
+        // Remaining partial tiles: padded to whole groups of pairs (2 lanes
+        // per body each) with massless sources far away.
         const float FAR = 1e18f;
-        if (pc_n > 0) {
-            const int s = pc_head + pc_n + lane;
-            if (lane < 32 - pc_n)
-                put_cell(R, s, make_float4(FAR, FAR, FAR, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float2(0.f, 0.f));
-            __syncwarp();
-            tile_pc<BPL, RPAIR>(lg, R.c0 + (pc_head >> 1), phase, me, eps2x2, A);
-        }
-        if (pp_n > 0) {
-            if (lane < 32 - pp_n) put_body(R, pp_head + pp_n + lane, make_float4(FAR, FAR, FAR, 0.f));
-            __syncwarp();
-            tile_pp<BPL, RPAIR>(lg, R.b0 + (pp_head >> 1), phase, me, eps2x2, A);
-        }
+        const int unit = 2 * (32 >> lg);                       // sources that the lanes of a body take at once
+        const int pad_c = -pc_n & (unit - 1), pad_b = -pp_n & (unit - 1);
+        if (lane < pad_c)
+            put_cell(R, ring_at(pc_head + pc_n + lane), make_float4(FAR, FAR, FAR, 0.f),
+                     make_float4(0.f, 0.f, 0.f, 0.f), make_float2(0.f, 0.f));
+        if (lane < pad_b) put_body(R, ring_at(pp_head + pp_n + lane), make_float4(FAR, FAR, FAR, 0.f));
+        __syncwarp();
+        if (pc_n > 0) tile_eval<true, BPL>(lg, R.c0, pc_head, pc_n + pad_c, phase, me, eps2x2, A);
+        if (pp_n > 0) tile_eval<false, BPL>(lg, R.b0, pp_head, pp_n + pad_b, phase, me, eps2x2, A);
 #pragma unroll
         for (int b = 0; b < BPL; b++) {
             float ax = A[b].ax - A[b].cx, ay = A[b].ay - A[b].cy, az = A[b].az - A[b].cz,
@@ -637,7 +610,7 @@ size_t walk_smem_bytes(int warps, int stack_cap) {
 // Function attribute and occupancy are set up once per shape, before any
 // stream capture of a step (the first step always runs eagerly).
 template <int BPL, bool FEAT, bool BLOCK>
-static cudaError_t launch_walk_t(Ctx &c, float eps, const unsigned *gate, bool three, cudaStream_t stream) {
+static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned *gate, bool three, cudaStream_t stream) {
     const unsigned polls = (unsigned)(c.max_spin < 0xffffffffll ? c.max_spin : 0xffffffffll);
     const int warps = c.walk_warps;
     const size_t smem = walk_smem_bytes(warps, c.list_capacity);
@@ -656,7 +629,7 @@ static cudaError_t launch_walk_t(Ctx &c, float eps, const unsigned *gate, bool t
         occ_warps[dv] = warps; occ_smem[dv] = smem; occ_per_sm[dv] = per < 1 ? 1 : per;
     }
     k_walk<BPL, FEAT, BLOCK><<<c.num_sms * occ_per_sm[dv], warps * 32, smem, stream>>>(
-        c.st, c.st, c.groups, c.pos4, c.test, c.cell_link, c.mono, c.quadA, c.quadB, c.sysid, eps,
+        c.st, c.st, c.groups, c.pos4, c.delta, 1.0f / theta, c.cell_link, c.mono, c.quadA, c.quadB, c.sysid, eps,
         c.list_capacity, polls, c.acc4, c.counts, c.cell_level, c.feat, gate,
         BLOCK ? c.vel4 : nullptr, c.block_s, c.block_kmax, three);
     return cudaGetLastError();
@@ -667,7 +640,7 @@ static cudaError_t launch_walk_t(Ctx &c, float eps, const unsigned *gate, bool t
 // With both, the two-body launch runs on a side stream forked from and
 // joined back into the context's stream (event edges inside a captured
 // step), so the tail of each launch overlaps the other's work.
-cudaError_t launch_walk(Ctx &c, float eps, bool features, const unsigned *gate) {
+cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features, const unsigned *gate) {
     // Second instantiation beside one body per lane: two bodies per lane for
     // groups of more than 32 bodies, or, in walks without learned features
     // and with groups of at most 32 bodies, three per lane for groups of
@@ -676,16 +649,16 @@ cudaError_t launch_walk(Ctx &c, float eps, bool features, const unsigned *gate) 
     // instantiations: plain, with learned features, or block time steps
     auto one = [&](int bpl, cudaStream_t st) -> cudaError_t {
         if (c.block_kmax >= 0) {
-            if (bpl == 3) return launch_walk_t<3, false, true>(c, eps, gate, true, st);
-            return bpl == 2 ? launch_walk_t<2, false, true>(c, eps, gate, false, st)
-                            : launch_walk_t<1, false, true>(c, eps, gate, three, st);
+            if (bpl == 3) return launch_walk_t<3, false, true>(c, theta, eps, gate, true, st);
+            return bpl == 2 ? launch_walk_t<2, false, true>(c, theta, eps, gate, false, st)
+                            : launch_walk_t<1, false, true>(c, theta, eps, gate, three, st);
         }
         if (features)
-            return bpl == 2 ? launch_walk_t<2, true, false>(c, eps, gate, false, st)
-                            : launch_walk_t<1, true, false>(c, eps, gate, false, st);
-        if (bpl == 3) return launch_walk_t<3, false, false>(c, eps, gate, true, st);
-        return bpl == 2 ? launch_walk_t<2, false, false>(c, eps, gate, false, st)
-                        : launch_walk_t<1, false, false>(c, eps, gate, three, st);
+            return bpl == 2 ? launch_walk_t<2, true, false>(c, theta, eps, gate, false, st)
+                            : launch_walk_t<1, true, false>(c, theta, eps, gate, false, st);
+        if (bpl == 3) return launch_walk_t<3, false, false>(c, theta, eps, gate, true, st);
+        return bpl == 2 ? launch_walk_t<2, false, false>(c, theta, eps, gate, false, st)
+                        : launch_walk_t<1, false, false>(c, theta, eps, gate, three, st);
     };
     const int second = c.ncrit >= WALK_BPL2_FROM ? 2 : three ? 3 : 0;
     if (second == 0) return one(1, c.stream);
