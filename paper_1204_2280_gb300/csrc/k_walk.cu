@@ -689,39 +689,87 @@ cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features, const uns
 // per group: two body slots per lane.
 namespace bonsai {
 
-constexpr int SPH_RING = 64;
+// Bound: instruction issue.  A ring of up to 64 candidates is taken in two
+// steps.  First every lane tests all of them against its body with packed
+// FP32x2 arithmetic, two candidates at a time, and keeps one bit each (six
+// instructions a candidate); then it runs over its own set bits only, about
+// one in six, and evaluates the kernel there.  Evaluating the kernel inside
+// the candidate loop instead made the whole warp take that path for nearly
+// every candidate: 24,600 warp instructions per group and 1402 us, 12,900 and 647
+// us now (2^20 bodies, 50 neighbours each, 430 candidates per group).
+constexpr int SPH_TILE = 64;                    // candidates evaluated together
+constexpr int SPH_RING = 128, SPH_RP = SPH_RING / 2;   // up to 63 waiting and a pass's 32
 
 struct SphWarp {
-    float4 src[SPH_RING];
+    float4 src[2][SPH_RP];      // source pairs: x x' y y' | z z' m m'
+    uint2 leaf[32];             // searched leaves of a round: first body, offset in the round's body list
 };
 
 // 8 / pi: the cubic spline's normalisation in three dimensions.
 constexpr float SPH_NORM = 2.546479089470325f;
 
-// One ring of sources: plain float32 sums per body, then one compensated
-// (Kahan) add into the body's density.
-__device__ __forceinline__ void sph_tile(const float4 *__restrict__ src, int nsrc, const float4 (&me)[2],
+// n <= 64 sources from place head (0 or 64; n padded to a multiple of 8):
+// plain float32 sums per body in source order, then one compensated (Kahan)
+// add into the body's density.
+template <int NB>
+__device__ __forceinline__ void sph_tile(const SphWarp &R, int head, int n, const float4 (&me)[2],
                                          const float (&h2)[2], const float (&ih)[2], const bool (&live)[2],
                                          float (&rho)[2], float (&comp)[2], unsigned (&cnt)[2]) {
-    float part[2] = {0.f, 0.f};
-    for (int k = 0; k < nsrc; k++) {
-        const float4 s = src[k];
+    const float4 *base = R.src[0] + (head >> 1);
 #pragma unroll
-        for (int b = 0; b < 2; b++) {
-            if (!live[b]) continue;
-            const float dx = __fsub_rn(s.x, me[b].x), dy = __fsub_rn(s.y, me[b].y), dz = __fsub_rn(s.z, me[b].z);
-            const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-            if (r2 < h2[b]) {
-                const float q = sqrtf(r2) * ih[b];
-                const float t = fmaxf(1.f - q, 0.f);
-                const float w = q <= 0.5f ? fmaf(6.f * q * q, q - 1.f, 1.f) : 2.f * t * t * t;
-                part[b] = fmaf(s.w, w, part[b]);
-                cnt[b]++;
+    for (int b = 0; b < NB; b++) {
+        const float2 nx = make_float2(-me[b].x, -me[b].x), ny = make_float2(-me[b].y, -me[b].y),
+                     nz = make_float2(-me[b].z, -me[b].z);
+        // r^2 < h^2 iff the difference (never rounded to zero) is negative:
+        // its sign bit is shifted into a mask, first source highest
+        const float2 nh = make_float2(-h2[b], -h2[b]);
+        unsigned in[2] = {0u, 0u};
+#pragma unroll
+        for (int half = 0; half < 2; half++) {
+            const int n_h = min(n - 32 * half, 32);
+            for (int k0 = 0; k0 < n_h; k0 += 8) {
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const int k = 16 * half + (k0 >> 1) + j;
+                    const float4 u = base[k], v = base[SPH_RP + k];
+                    const float2 dx = __fadd2_rn(make_float2(u.x, u.y), nx),
+                                 dy = __fadd2_rn(make_float2(u.z, u.w), ny),
+                                 dz = __fadd2_rn(make_float2(v.x, v.y), nz);
+                    const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+                    const float2 d = __fadd2_rn(r2, nh);
+                    in[half] = __funnelshift_l(__float_as_uint(d.x), in[half], 1);
+                    in[half] = __funnelshift_l(__float_as_uint(d.y), in[half], 1);
+                }
             }
+            if (n_h < 32) in[half] = n_h > 0 ? in[half] << (32 - n_h) : 0u;
         }
+        if (!live[b]) in[0] = in[1] = 0u;
+        cnt[b] += (unsigned)(__popc(in[0]) + __popc(in[1]));
+        float part = 0.f;
+        while (in[0] | in[1]) {
+            const bool first = in[0] != 0u;
+            const int z = __clz((int)(first ? in[0] : in[1]));
+            const unsigned bit = 0x80000000u >> z;
+            const int k = first ? z : 32 + z;
+            if (first) in[0] ^= bit; else in[1] ^= bit;
+            const float *f = reinterpret_cast<const float *>(base + (k >> 1)) + (k & 1);
+            const float *g = f + 4 * SPH_RP;
+            const float dx = __fsub_rn(f[0], me[b].x), dy = __fsub_rn(f[2], me[b].y), dz = __fsub_rn(g[0], me[b].z);
+            const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+            const float q = sqrtf(r2) * ih[b];
+            const float t = fmaxf(1.f - q, 0.f);
+            const float w = q <= 0.5f ? fmaf(6.f * q * q, q - 1.f, 1.f) : 2.f * t * t * t;
+            part = fmaf(g[2], w, part);
+        }
+        kahan_add(rho[b], comp[b], part);
     }
-#pragma unroll
-    for (int b = 0; b < 2; b++) kahan_add(rho[b], comp[b], part[b]);
+}
+
+__device__ __forceinline__ void sph_eval(bool two, const SphWarp &R, int head, int n, const float4 (&me)[2],
+                                         const float (&h2)[2], const float (&ih)[2], const bool (&live)[2],
+                                         float (&rho)[2], float (&comp)[2], unsigned (&cnt)[2]) {
+    if (two) sph_tile<2>(R, head, n, me, h2, ih, live, rho, comp, cnt);
+    else sph_tile<1>(R, head, n, me, h2, ih, live, rho, comp, cnt);
 }
 
 __global__ void __launch_bounds__(128)
@@ -777,7 +825,7 @@ k_sph_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restri
         }
         // search radius with a relative slack: rounding may only open more
         const float reach2 = hmax * hmax * 1.0001f;
-        int sp = 1, nsrc = 0;
+        int sp = 1, nsrc = 0, head = 0;
         if (lane == 0) stk[0] = (unsigned)sysid[gb] << 3;   // the root of the group's system
         bool overflow = false, timeout = false;
         unsigned rounds = 0;
@@ -806,40 +854,59 @@ k_sph_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restri
                 if (open && !isleaf) stk[sp + __popc(im & lt)] = (lk.x << 3) | ((lk.y - 1u) & 7u);
                 sp += np;
             }
-            // searched leaves, one at a time: their bodies into the ring
-            unsigned lm = __ballot_sync(0xffffffffu, open && isleaf);
-            while (lm) {
-                const int src_lane = __ffs(lm) - 1;
-                lm &= lm - 1;
-                const unsigned first = __shfl_sync(0xffffffffu, lk.x, src_lane);
-                const int n_l = (int)(__shfl_sync(0xffffffffu, lk.y, src_lane) & ~LEAF_BIT);
-                for (int off = 0; off < n_l; off += 32) {
-                    // a body farther than h_max from the group's box is no
-                    // body's neighbour: only the others enter the ring
+            // searched leaves: the bodies of all of the round's, in lane
+            // order, 32 per pass; a body farther than h_max from the group's
+            // box is no body's neighbour: only the others enter the ring
+            const bool ol = open && isleaf;
+            const unsigned lm = __ballot_sync(0xffffffffu, ol);
+            if (lm) {
+                const unsigned lc = ol ? (lk.y & ~LEAF_BIT) : 0u;
+                unsigned lincl = lc;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, lincl, o);
+                    if (lane >= o) lincl += y;
+                }
+                const unsigned total = __shfl_sync(0xffffffffu, lincl, 31);
+                const unsigned lex = lincl - lc;
+                if (ol) R.leaf[__popc(lm & lt)] = make_uint2(lk.x, lex);
+                __syncwarp();
+                const unsigned upto = 0xffffffffu >> (31 - lane);
+                for (unsigned base = 0; base < total; base += 32u) {
+                    const unsigned starts =
+                        __reduce_or_sync(0xffffffffu, ol && lex >= base && lex < base + 32u ? 1u << (lex - base) : 0u);
+                    const int before = __popc(__ballot_sync(0xffffffffu, ol && lex < base));
+                    const uint2 li = R.leaf[before + __popc(starts & upto) - 1];
                     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
                     bool keep = false;
-                    if (off + lane < n_l) {
-                        p = __ldg(pos4 + first + off + lane);
+                    if (base + lane < total) {
+                        p = __ldg(pos4 + li.x + (base + lane - li.y));
                         const float ex = fmaxf(fmaxf(bx0 - p.x, p.x - bx1), 0.f);
                         const float ey = fmaxf(fmaxf(by0 - p.y, p.y - by1), 0.f);
                         const float ez = fmaxf(fmaxf(bz0 - p.z, p.z - bz1), 0.f);
                         keep = fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= reach2;
                     }
                     const unsigned km = __ballot_sync(0xffffffffu, keep);
-                    const int take = __popc(km);
-                    if (nsrc + take > SPH_RING) {           // ring full: evaluate it
+                    if (keep)
+                        put_body_at<SPH_RP>(R.src[0], (head + nsrc + __popc(km & lt)) & (SPH_RING - 1), p);
+                    nsrc += __popc(km);
+                    if (nsrc >= SPH_TILE) {
                         __syncwarp();
-                        sph_tile(R.src, nsrc, me, h2, ih, live, rho, comp, cnt);
+                        sph_eval(ng > 32, R, head, SPH_TILE, me, h2, ih, live, rho, comp, cnt);
                         __syncwarp();
-                        nsrc = 0;
+                        head = (head + SPH_TILE) & (SPH_RING - 1);
+                        nsrc -= SPH_TILE;
                     }
-                    if (keep) R.src[nsrc + __popc(km & lt)] = p;
-                    nsrc += take;
                 }
             }
             __syncwarp();
         }
-        if (nsrc > 0) sph_tile(R.src, nsrc, me, h2, ih, live, rho, comp, cnt);
+        if (nsrc > 0) {
+            const int pad = -nsrc & 7;                  // sources far away, no body's neighbours
+            if (lane < pad) put_body_at<SPH_RP>(R.src[0], head + nsrc + lane, make_float4(1e18f, 1e18f, 1e18f, 0.f));
+            __syncwarp();
+            sph_eval(ng > 32, R, head, nsrc + pad, me, h2, ih, live, rho, comp, cnt);
+        }
 #pragma unroll
         for (int b = 0; b < 2; b++) {
             if (live[b]) {

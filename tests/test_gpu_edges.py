@@ -91,3 +91,24 @@ def test_build_order_across_sorts(n):
             B.bonsai_get_bodies(bz.ctx, x, v)
             assert np.array_equal(x, pos) and np.array_equal(v, pos)
         bz.sync()
+
+
+@pytest.mark.parametrize("n,ncrit", [(1, 32), (7, 32), (9, 64), (63, 64), (65, 32), (129, 64), (200, 16), (700, 64)])
+def test_sph_candidate_rings(n, ncrit):
+    """Neighbour counts and densities where the candidates end inside, at and
+    past the 64-source ring: every body a neighbour of every other, and about
+    half of them.  Counts are decided in FP32 as the oracle decides them;
+    densities are sums of up to n FP32 terms in chains of at most 64 with
+    compensated adds: within 2e-5."""
+    import oracle
+    rng = np.random.default_rng(n)
+    pos = rng.normal(size=(n, 3)).astype(np.float32)
+    mass = rng.uniform(0.5, 1.5, n).astype(np.float32)
+    for h in (np.full(n, 50.0, np.float32), rng.uniform(1.0, 2.5, n).astype(np.float32)):
+        rho, cnt = np.zeros(n, np.float32), np.zeros(n, np.int32)
+        with B.Bonsai(B.Config(ncrit=ncrit)) as bz:
+            bz.set_bodies(pos, mass).build()
+            B.bonsai_sph_density(bz.ctx, h, rho, cnt)
+            bz.sync()
+        ref = oracle.sph_density(pos, mass, h)
+        assert np.array_equal(cnt, ref[1]) and np.abs(rho / ref[0] - 1.0).max() <= 2e-5
