@@ -112,3 +112,41 @@ def test_sph_candidate_rings(n, ncrit):
             bz.sync()
         ref = oracle.sph_density(pos, mass, h)
         assert np.array_equal(cnt, ref[1]) and np.abs(rho / ref[0] - 1.0).max() <= 2e-5
+
+
+@pytest.mark.parametrize("n", [(1 << 18) - 1, 1 << 18, (1 << 18) + 1, 300001])
+def test_caller_order_outputs(n):
+    """Positions, velocities, forces and potentials in caller order on both
+    sides of the gather's size rule, each output alone and together, device
+    and host: loaded values come back bit for bit, forces equal the sorted
+    ones through the permutation."""
+    import torch
+    rng = np.random.default_rng(n)
+    pos, vel = (rng.normal(size=(n, 3)).astype(np.float32) for _ in range(2))
+    mass = np.full(n, 1.0 / n, np.float32)
+    with B.Bonsai(B.Config(ncrit=32, group_pack=1)) as bz:
+        bz.set_bodies(pos, mass, vel).build().multipoles()
+        x, v = (torch.zeros(n, 3, device="cuda") for _ in range(2))
+        B.bonsai_get_bodies(bz.ctx, x, v)
+        assert np.array_equal(x.cpu().numpy(), pos) and np.array_equal(v.cpu().numpy(), vel)
+        v.zero_()
+        B.bonsai_get_bodies(bz.ctx, None, v)
+        assert np.array_equal(v.cpu().numpy(), vel)
+        hx = np.zeros((n, 3), np.float32)
+        B.bonsai_get_bodies(bz.ctx, hx, None)
+        assert np.array_equal(hx, pos)
+        acc, pot = torch.zeros(n, 3, device="cuda"), torch.zeros(n, device="cuda")
+        bz.forces(1.0, 0.01, acc, pot)
+        both = acc.cpu().numpy(), pot.cpu().numpy()
+        alone = np.zeros((n, 3), np.float32), np.zeros(n, np.float32)
+        bz.forces(1.0, 0.01, alone[0], None)
+        bz.forces(1.0, 0.01, None, alone[1])
+        bz.sync()
+        assert np.array_equal(both[0], alone[0]) and np.array_equal(both[1], alone[1])
+    # the scatter's route: potentials alone; a rotated order of the same bodies
+    perm = np.roll(np.arange(n), 12345)
+    with B.Bonsai(B.Config(ncrit=32, group_pack=1)) as bz:
+        a2, p2 = torch.zeros(n, 3, device="cuda"), torch.zeros(n, device="cuda")
+        bz.set_bodies(pos[perm], mass, vel[perm]).build().multipoles().forces(1.0, 0.01, a2, p2)
+        bz.sync()
+        assert np.array_equal(a2.cpu().numpy(), both[0][perm]) and np.array_equal(p2.cpu().numpy(), both[1][perm])
