@@ -97,7 +97,14 @@ __device__ __forceinline__ void body_features(const float4 a, const float *__res
 }
 
 // ---------------------------------------------------------------------------
-// Inference on tensor cores.  One warp per 16 bodies.
+// Inference on tensor cores.  One warp per 32 bodies: every lane forms the
+// inputs and the frame of its own body, the two 16-row halves share each
+// weight fragment read from shared memory, whose rows are padded so that the
+// eight rows of a fragment fall in different banks.  Bound: the per-body
+// input arithmetic (two logarithms, four roots, ten divisions) and latency.
+// With 16 lanes forming inputs, rows of 32 words (eight-way conflicts on
+// every weight read) and the frames in shared memory 2^20 bodies took 191 us,
+// 62 us now.
 // ---------------------------------------------------------------------------
 constexpr int INF_WARPS = 4;
 
@@ -111,15 +118,15 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 
 // Weights as BF16 pairs in shared memory: W1 64 x 16 (inputs padded to 16),
 // W2 64 x 64, W3 8 x 64 (outputs padded to 8); row n holds W[n][k..].
+constexpr int LD1 = 12, LD2 = 36;   // row strides in words: 12 g + t and 36 g + t are 32 different banks
 struct InfShared {
-    uint32_t w1[MLP_H * 8];
-    uint32_t w2[MLP_H * 32];
-    uint32_t w3[8 * 32];
+    uint32_t w1[MLP_H * LD1];
+    uint32_t w2[MLP_H * LD2];
+    uint32_t w3[8 * LD2];
     float b1[MLP_H], b2[MLP_H], b3[8];
     float norm[2 * MLP_IN], ysig;
-    float xs[INF_WARPS][16][17];
-    float ys[INF_WARPS][16][4];
-    float fr[INF_WARPS][16][10];     // frame e0 e1 e2 and |a| of each row
+    float xs[INF_WARPS][32][17];
+    float ys[INF_WARPS][32][5];
 };
 
 __device__ void stage_weights(InfShared &S, const float *__restrict__ P, const float *__restrict__ norm) {
@@ -128,15 +135,16 @@ __device__ void stage_weights(InfShared &S, const float *__restrict__ P, const f
         const int r = i / 8, c = 2 * (i % 8);
         const float a = c < MLP_IN ? P[OFF_W1 + r * MLP_IN + c] : 0.f;
         const float b = c + 1 < MLP_IN ? P[OFF_W1 + r * MLP_IN + c + 1] : 0.f;
-        S.w1[i] = pack_bf16(a, b);
+        S.w1[r * LD1 + i % 8] = pack_bf16(a, b);
     }
+#pragma unroll 8
     for (int i = tid; i < MLP_H * 32; i += blockDim.x) {
         const int r = i / 32, c = 2 * (i % 32);
-        S.w2[i] = pack_bf16(P[OFF_W2 + r * MLP_H + c], P[OFF_W2 + r * MLP_H + c + 1]);
+        S.w2[r * LD2 + i % 32] = pack_bf16(P[OFF_W2 + r * MLP_H + c], P[OFF_W2 + r * MLP_H + c + 1]);
     }
     for (int i = tid; i < 8 * 32; i += blockDim.x) {
         const int r = i / 32, c = 2 * (i % 32);
-        S.w3[i] = r < MLP_OUT ? pack_bf16(P[OFF_W3 + r * MLP_H + c], P[OFF_W3 + r * MLP_H + c + 1]) : 0u;
+        S.w3[r * LD2 + i % 32] = r < MLP_OUT ? pack_bf16(P[OFF_W3 + r * MLP_H + c], P[OFF_W3 + r * MLP_H + c + 1]) : 0u;
     }
     for (int i = tid; i < MLP_H; i += blockDim.x) { S.b1[i] = P[OFF_B1 + i]; S.b2[i] = P[OFF_B2 + i]; }
     if (tid < 8) S.b3[tid] = tid < MLP_OUT ? P[OFF_B3 + tid] : 0.f;
@@ -154,39 +162,62 @@ __device__ __forceinline__ void relu_pack(const float (&h)[8][4], uint32_t (&a2)
     }
 }
 
-// Forward of 16 rows (normalised inputs xs[16][<=16]) on the tensor cores;
-// the raw outputs land in ys[16][0..2].  Whole warp.
-__device__ void mma_forward16(const InfShared &S, const float (*xs)[17], float (*ys)[4], int lane) {
+// Forward of 32 rows (normalised inputs xs[32][<=16]) on the tensor cores;
+// the raw outputs land in ys[32][0..2].  Whole warp.
+__device__ __forceinline__ void mma_forward32(const InfShared &S, const float (*xs)[17], float (*ys)[5], int lane) {
     const int g = lane >> 2, t = lane & 3;
-    uint32_t a[4] = {pack_bf16(xs[g][2 * t], xs[g][2 * t + 1]), pack_bf16(xs[g + 8][2 * t], xs[g + 8][2 * t + 1]),
-                     pack_bf16(xs[g][2 * t + 8], xs[g][2 * t + 9]),
-                     pack_bf16(xs[g + 8][2 * t + 8], xs[g + 8][2 * t + 9])};
-    float h[8][4];
+    uint32_t a[2][4], a2[2][4][4];
+    float h[2][8][4];
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+        const float *x0 = xs[16 * r + g], *x1 = xs[16 * r + g + 8];
+        a[r][0] = pack_bf16(x0[2 * t], x0[2 * t + 1]); a[r][1] = pack_bf16(x1[2 * t], x1[2 * t + 1]);
+        a[r][2] = pack_bf16(x0[2 * t + 8], x0[2 * t + 9]); a[r][3] = pack_bf16(x1[2 * t + 8], x1[2 * t + 9]);
+    }
 #pragma unroll
     for (int j = 0; j < 8; j++) {                 // layer 1: 8 n-tiles of 8 hidden units
         const int col = 8 * j + 2 * t, row = 8 * j + g;
-        h[j][0] = S.b1[col]; h[j][1] = S.b1[col + 1]; h[j][2] = S.b1[col]; h[j][3] = S.b1[col + 1];
-        mma_bf16(h[j], a, S.w1[row * 8 + t], S.w1[row * 8 + t + 4]);
+        const float c0 = S.b1[col], c1 = S.b1[col + 1];
+        const uint32_t w0 = S.w1[row * LD1 + t], w1 = S.w1[row * LD1 + t + 4];
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            h[r][j][0] = c0; h[r][j][1] = c1; h[r][j][2] = c0; h[r][j][3] = c1;
+            mma_bf16(h[r][j], a[r], w0, w1);
+        }
     }
-    uint32_t a2[4][4];
-    relu_pack(h, a2);                             // accumulator layout == next A layout
+    relu_pack(h[0], a2[0]);                       // accumulator layout == next A layout
+    relu_pack(h[1], a2[1]);
 #pragma unroll
     for (int j = 0; j < 8; j++) {                 // layer 2
         const int col = 8 * j + 2 * t, row = 8 * j + g;
-        h[j][0] = S.b2[col]; h[j][1] = S.b2[col + 1]; h[j][2] = S.b2[col]; h[j][3] = S.b2[col + 1];
+        const float c0 = S.b2[col], c1 = S.b2[col + 1];
 #pragma unroll
-        for (int kc = 0; kc < 4; kc++)
-            mma_bf16(h[j], a2[kc], S.w2[row * 32 + 8 * kc + t], S.w2[row * 32 + 8 * kc + t + 4]);
-    }
-    relu_pack(h, a2);
-    float y[4] = {S.b3[2 * t], S.b3[2 * t + 1], S.b3[2 * t], S.b3[2 * t + 1]};
+        for (int r = 0; r < 2; r++) { h[r][j][0] = c0; h[r][j][1] = c1; h[r][j][2] = c0; h[r][j][3] = c1; }
 #pragma unroll
-    for (int kc = 0; kc < 4; kc++)                // layer 3 (outputs padded to 8)
-        mma_bf16(y, a2[kc], S.w3[g * 32 + 8 * kc + t], S.w3[g * 32 + 8 * kc + t + 4]);
-    if (t < 2) {
-        ys[g][2 * t] = y[0]; ys[g][2 * t + 1] = y[1];
-        ys[g + 8][2 * t] = y[2]; ys[g + 8][2 * t + 1] = y[3];
+        for (int kc = 0; kc < 4; kc++) {
+            const uint32_t w0 = S.w2[row * LD2 + 8 * kc + t], w1 = S.w2[row * LD2 + 8 * kc + t + 4];
+#pragma unroll
+            for (int r = 0; r < 2; r++) mma_bf16(h[r][j], a2[r][kc], w0, w1);
+        }
     }
+    relu_pack(h[0], a2[0]);
+    relu_pack(h[1], a2[1]);
+    float y[2][4];
+#pragma unroll
+    for (int r = 0; r < 2; r++) { y[r][0] = S.b3[2 * t]; y[r][1] = S.b3[2 * t + 1]; y[r][2] = y[r][0]; y[r][3] = y[r][1]; }
+#pragma unroll
+    for (int kc = 0; kc < 4; kc++) {              // layer 3 (outputs padded to 8)
+        const uint32_t w0 = S.w3[g * LD2 + 8 * kc + t], w1 = S.w3[g * LD2 + 8 * kc + t + 4];
+#pragma unroll
+        for (int r = 0; r < 2; r++) mma_bf16(y[r], a2[r][kc], w0, w1);
+    }
+    if (t < 2)
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            float *y0 = ys[16 * r + g], *y1 = ys[16 * r + g + 8];
+            y0[2 * t] = y[r][0]; y0[2 * t + 1] = y[r][1];
+            y1[2 * t] = y[r][2]; y1[2 * t + 1] = y[r][3];
+        }
 }
 
 // Corrects the tree accelerations in place: a += ysig |a| (y0 e0 + y1 e1 + y2 e2).
@@ -198,38 +229,37 @@ k_mlp_infer(const float *__restrict__ P, const float *__restrict__ norm, float4 
     if (st->status & ST_TIMEOUT) return;
     stage_weights(S, P, norm);
     __syncthreads();
-    const int nwarps_total = gridDim.x * INF_WARPS;
-    for (int base = (blockIdx.x * INF_WARPS + warp) * 16; base < n; base += nwarps_total * 16) {
-        if (lane < 16) {
-            const int i = base + lane;
-            float x[MLP_IN];
-            Frame F{};
-            if (i < n) {
-                body_features(acc4[i], feat + FEAT_STRIDE * (size_t)i, S.norm, x, F);
-            } else {
+    const int step = gridDim.x * INF_WARPS * 32;
+    for (int base = (blockIdx.x * INF_WARPS + warp) * 32; base < n; base += step) {
+        const int i = base + lane;
+        float4 av = make_float4(0.f, 0.f, 0.f, 0.f);
+        float x[MLP_IN];
+        Frame F{};
+        if (i < n) {
+            av = acc4[i];
+            float f[FEAT_STRIDE];                 // a row of features is three aligned 16-byte words
+            const float4 *fp = reinterpret_cast<const float4 *>(feat + FEAT_STRIDE * (size_t)i);
 #pragma unroll
-                for (int k = 0; k < MLP_IN; k++) x[k] = 0.f;
+            for (int q = 0; q < 3; q++) {
+                const float4 v = fp[q];
+                f[4 * q] = v.x; f[4 * q + 1] = v.y; f[4 * q + 2] = v.z; f[4 * q + 3] = v.w;
             }
-            float *fr = S.fr[warp][lane];
-            fr[0] = F.e0.x; fr[1] = F.e0.y; fr[2] = F.e0.z; fr[3] = F.e1.x; fr[4] = F.e1.y;
-            fr[5] = F.e1.z; fr[6] = F.e2.x; fr[7] = F.e2.y; fr[8] = F.e2.z; fr[9] = F.an;
+            body_features(av, f, S.norm, x, F);
+        } else {
 #pragma unroll
-            for (int k = 0; k < MLP_IN; k++) S.xs[warp][lane][k] = x[k];
-#pragma unroll
-            for (int k = MLP_IN; k < 16; k++) S.xs[warp][lane][k] = 0.f;
+            for (int k = 0; k < MLP_IN; k++) x[k] = 0.f;
         }
+#pragma unroll
+        for (int k = 0; k < 16; k++) S.xs[warp][lane][k] = k < MLP_IN ? x[k] : 0.f;
         __syncwarp();
-        mma_forward16(S, S.xs[warp], S.ys[warp], lane);
+        mma_forward32(S, S.xs[warp], S.ys[warp], lane);
         __syncwarp();
-        if (lane < 16 && base + lane < n) {
-            const int i = base + lane;
-            float4 av = acc4[i];
-            const float *fr = S.fr[warp][lane];
-            const float s = fr[9] * S.ysig;
+        if (i < n) {
+            const float s = F.an * S.ysig;
             const float c0 = S.ys[warp][lane][0] * s, c1 = S.ys[warp][lane][1] * s, c2 = S.ys[warp][lane][2] * s;
-            av.x += c0 * fr[0] + c1 * fr[3] + c2 * fr[6];
-            av.y += c0 * fr[1] + c1 * fr[4] + c2 * fr[7];
-            av.z += c0 * fr[2] + c1 * fr[5] + c2 * fr[8];
+            av.x += c0 * F.e0.x + c1 * F.e1.x + c2 * F.e2.x;
+            av.y += c0 * F.e0.y + c1 * F.e1.y + c2 * F.e2.y;
+            av.z += c0 * F.e0.z + c1 * F.e1.z + c2 * F.e2.z;
             acc4[i] = av;
         }
         __syncwarp();
@@ -244,21 +274,19 @@ k_mlp_rows(const float *__restrict__ P, const float *__restrict__ norm, const fl
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     stage_weights(S, P, norm);
     __syncthreads();
-    const int nwarps_total = gridDim.x * INF_WARPS;
-    for (int base = (blockIdx.x * INF_WARPS + warp) * 16; base < n; base += nwarps_total * 16) {
-        if (lane < 16) {
-            const int i = base + lane;
+    const long long step = (long long)gridDim.x * INF_WARPS * 32;
+    for (long long base = (blockIdx.x * INF_WARPS + warp) * 32; base < n; base += step) {
+        const long long i = base + lane;
 #pragma unroll
-            for (int k = 0; k < 16; k++)
-                S.xs[warp][lane][k] = (k < MLP_IN && i < n)
-                                          ? (X[(size_t)i * MLP_IN + k] - S.norm[k]) / S.norm[MLP_IN + k]
-                                          : 0.f;
-        }
+        for (int k = 0; k < 16; k++)
+            S.xs[warp][lane][k] = (k < MLP_IN && i < n)
+                                      ? (X[(size_t)i * MLP_IN + k] - S.norm[k]) / S.norm[MLP_IN + k]
+                                      : 0.f;
         __syncwarp();
-        mma_forward16(S, S.xs[warp], S.ys[warp], lane);
+        mma_forward32(S, S.xs[warp], S.ys[warp], lane);
         __syncwarp();
-        if (lane < 16 && base + lane < n)
-            for (int o = 0; o < MLP_OUT; o++) Y[(size_t)(base + lane) * MLP_OUT + o] = S.ys[warp][lane][o];
+        if (i < n)
+            for (int o = 0; o < MLP_OUT; o++) Y[(size_t)i * MLP_OUT + o] = S.ys[warp][lane][o];
         __syncwarp();
     }
 }
@@ -568,7 +596,7 @@ k_adamw(float *P, const float *__restrict__ part, int nblk, float *m, float *v, 
 
 cudaError_t launch_mlp_infer(Ctx &c, const float *P, const float *norm) {
     const int n = (int)c.n;
-    int blocks = (n + INF_WARPS * 16 - 1) / (INF_WARPS * 16);
+    int blocks = (n + INF_WARPS * 32 - 1) / (INF_WARPS * 32);
     const int cap = c.num_sms * 8;
     if (blocks > cap) blocks = cap;
     k_mlp_infer<<<blocks, INF_WARPS * 32, 0, c.stream>>>(P, norm, c.acc4, c.feat, n, c.st);
@@ -576,7 +604,7 @@ cudaError_t launch_mlp_infer(Ctx &c, const float *P, const float *norm) {
 }
 
 cudaError_t launch_mlp_rows(cudaStream_t s, const float *P, const float *norm, const float *X, float *Y, int n) {
-    int blocks = (n + INF_WARPS * 16 - 1) / (INF_WARPS * 16);
+    int blocks = (n + INF_WARPS * 32 - 1) / (INF_WARPS * 32);
     if (blocks > 1216) blocks = 1216;
     k_mlp_rows<<<blocks, INF_WARPS * 32, 0, s>>>(P, norm, X, Y, n);
     return cudaGetLastError();
