@@ -150,3 +150,41 @@ def test_caller_order_outputs(n):
         bz.set_bodies(pos[perm], mass, vel[perm]).build().multipoles().forces(1.0, 0.01, a2, p2)
         bz.sync()
         assert np.array_equal(a2.cpu().numpy(), both[0][perm]) and np.array_equal(p2.cpu().numpy(), both[1][perm])
+
+
+@pytest.mark.parametrize("n", [1, 16, 31, 33, 127, 129, 5000])
+def test_network_rows(n):
+    """Inference of 32-row warp tiles against the FP64 oracle on the same
+    BF16-rounded weights: within 1e-2 of the output scale (BF16 ties)."""
+    rng = np.random.default_rng(n)
+    X = rng.normal(size=(n, B.MLP_IN)).astype(np.float32)
+    net = B.MLP(11)
+    P, norm = net.get_params()
+    y = net.predict(X)
+    ref, _ = OM.forward(P, norm, X)
+    assert np.abs(y - ref).max() <= 1e-2 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 101, 513, 4095, 4097, 30001])
+def test_judge_sizes(n):
+    """The judge at sizes around its target blocks and source splits: p99
+    against numpy's percentile of the oracle's direct sum, 1e-4 relative (the
+    FP32 error of both sums, 1e-7, against errors of at least 1e-3 of it)."""
+    import oracle
+    rng = np.random.default_rng(n)
+    pos = rng.normal(size=(n, 3)).astype(np.float32)
+    mass = np.full(n, 1.0 / n, np.float32)
+    acc = np.zeros((n, 3), np.float32)
+    with B.Bonsai(B.Config(ncrit=64)) as bz:
+        bz.set_bodies(pos, mass).build().multipoles()
+        bz.forces(1.1, 0.05, acc)
+        p = B.bonsai_judge(bz.ctx, 0.05)
+        _, perm = B.bonsai_get_keys(bz.ctx)
+        bz.sync()
+    t = min(n, 4096)
+    ids = perm[(np.arange(t, dtype=np.int64) * n) // t].astype(np.int64)
+    a, _ = oracle.direct(pos, mass, 0.05, ids)
+    norm = np.linalg.norm(a, axis=1)
+    e = np.where(norm > 0, np.linalg.norm(acc[ids] - a, axis=1) / np.maximum(norm, 1e-300), 0.0)
+    ref = np.percentile(e, 99)
+    assert abs(p - ref) <= 1e-4 * ref + 1e-6
