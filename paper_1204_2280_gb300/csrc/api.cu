@@ -88,7 +88,7 @@ cudaError_t alloc_bodies(Ctx &c, long long n) {
     a.take(c.group_lvl, n, plan); a.take(c.group_flag, n, plan); a.take(c.group_bcount, (n + PACK_THREADS - 1) / PACK_THREADS, plan);
     a.take(c.counts, n, plan); a.take(c.feat, FEAT_STRIDE * (size_t)n, plan);
     const long long stage_floats = 7 * n > STAGE_MIN_FLOATS ? 7 * n : STAGE_MIN_FLOATS;
-    a.take(c.stage, (size_t)stage_floats, plan);
+    a.take(c.stage, (size_t)stage_floats, plan); a.take(c.pack_box, 6 * (size_t)PACK_BLOCKS, plan);
     a.take(c.judge_targets, JUDGE_MAX, plan); a.take(c.judge_direct, JUDGE_MAX, plan);
     a.take(c.judge_partial, (size_t)JUDGE_SPLIT * JUDGE_MAX, plan);
     char *base = nullptr;
@@ -155,6 +155,15 @@ cudaError_t run_cached(Ctx &c, CallGraph &g, const long long *key, int nkey, F b
     for (int i = 0; i < nkey; i++) g.key[i] = key[i];
     g.nkey = nkey;
     return body();
+}
+
+// Whether the caller is capturing the stream: what a call may skip because an
+// earlier call has done it must then be in the captured launches all the
+// same, since they are replayed without that call.
+bool caller_captures(Ctx &c) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c.stream, &cs) != cudaSuccess) { cudaGetLastError(); return true; }
+    return cs != cudaStreamCaptureStatusNone;
 }
 
 long long fbits(float x) {
@@ -285,6 +294,7 @@ int bonsai_set_bodies(bonsai_ctx *ctx, const float *pos, const float *mass, cons
         if (e != cudaSuccess) {
             // the old arena is gone: the context holds no bodies now
             c.n = 0;
+            c.dom_ready = c.walk_ready = false;
             c.have_bodies = c.built = c.moments_ready = c.have_acc = c.tree_fresh = c.timed_step = false;
             c.graph_n = -1;
             return fail(ctx, e == cudaErrorMemoryAllocation ? BONSAI_ERR_OOM : BONSAI_ERR_CUDA,
@@ -319,16 +329,14 @@ int bonsai_set_bodies(bonsai_ctx *ctx, const float *pos, const float *mass, cons
         if (vel) CK(cudaMemcpyAsync(s + 4 * n, vel, 12 * (size_t)n, cudaMemcpyHostToDevice, c.stream));
         p = s; m = s + 3 * n; v = vel ? s + 4 * n : nullptr;
     }
-    CK(launch_pack(c, p, m, v));
     // One system holding every body until bonsai_set_systems says otherwise.
     c.nsys = 1;
-    unsigned off1[2] = {0u, (unsigned)n};
-    CK(cudaMemcpyAsync(c.st->sys_off, off1, sizeof(off1), cudaMemcpyHostToDevice, c.stream));
-    CK(cudaMemsetAsync(c.sysid, 0, (size_t)n, c.stream));
+    CK(launch_pack(c, p, m, v));
     CK(cudaStreamSynchronize(c.stream));
     // The state now lives in the pre-sort (*_alt) arrays; nothing derived
     // from earlier bodies stays valid.
-    c.have_bodies = true;
+    c.have_bodies = c.dom_ready = true;
+    c.walk_ready = false;
     c.built = c.moments_ready = c.have_acc = false;
     c.err.clear();
     return BONSAI_OK;
@@ -353,6 +361,7 @@ int bonsai_set_systems(bonsai_ctx *ctx, const long long *offsets, int nsys) {
     if (c.step_graph) { cudaGraphExecDestroy(c.step_graph); c.step_graph = nullptr; }
     c.graph_n = -1;
     c.nsys = nsys;
+    c.dom_ready = nsys == 1;
     CK(cudaMemcpyAsync(c.st->sys_off, off.data(), sizeof(unsigned) * (nsys + 1), cudaMemcpyHostToDevice,
                        c.stream));
     CK(launch_fill_sysid(c));
@@ -365,9 +374,9 @@ int bonsai_build(bonsai_ctx *ctx) {
     if (!ctx) return BONSAI_ERR_INVALID_ARG;
     Ctx &c = ctx->c;
     if (!c.have_bodies) return fail(ctx, BONSAI_ERR_NOT_READY, "bonsai_build: no bodies");
-    const bool again = c.built;
+    const bool again = c.built, boxed = c.dom_ready && !caller_captures(c);
     const long long key[] = {c.n, c.arena_gen, c.nsys, c.nleaf, c.ncrit, c.group_pack, c.max_spin, again,
-                             c.hold_tile};
+                             c.hold_tile, boxed};
     CK(run_cached(c, c.build_graph, key, (int)(sizeof key / sizeof key[0]), [&]() -> cudaError_t {
         cudaError_t e;
         if (again) {
@@ -379,10 +388,14 @@ int bonsai_build(bonsai_ctx *ctx) {
             if ((e = cudaMemcpyAsync(c.id_alt, c.id, 4 * (size_t)c.n, cudaMemcpyDeviceToDevice, c.stream)))
                 return e;
         }
-        if ((e = launch_reset(c)) != cudaSuccess) return e;
-        if ((e = launch_bbox(c)) != cudaSuccess) return e;
+        // set_bodies leaves the domain box of the first build; the merge sort
+        // keeps no counts
+        const int what = (boxed ? 0 : RESET_DOMAIN) | (sort_by_merge(c) ? 0 : RESET_SORT);
+        if (what && (e = launch_reset(c, what)) != cudaSuccess) return e;
+        if (!boxed && (e = launch_bbox(c)) != cudaSuccess) return e;
         return pipeline_tree(c);
     }));
+    c.dom_ready = false;
     c.built = c.tree_fresh = true;
     c.moments_ready = c.have_acc = false;
     return BONSAI_OK;
@@ -395,8 +408,11 @@ int bonsai_multipoles(bonsai_ctx *ctx) {
     // The launch is sized from the last known cell count (a tree of the same
     // bodies changes little); only a context without one reads it back.
     if (c.cells_hint == 0) CK(refresh_cells_hint(c));
-    const long long key[] = {c.n, c.arena_gen, c.nsys, c.cells_hint};
-    CK(run_cached(c, c.mom_graph, key, (int)(sizeof key / sizeof key[0]), [&]() { return launch_multipoles(c); }));
+    // the totals of a walk stay readable until the next one
+    const bool reset = !c.have_acc;
+    const long long key[] = {c.n, c.arena_gen, c.nsys, c.cells_hint, reset};
+    CK(run_cached(c, c.mom_graph, key, (int)(sizeof key / sizeof key[0]), [&]() { return launch_multipoles(c, reset); }));
+    c.walk_ready = reset;
     c.moments_ready = true;
     return BONSAI_OK;
 }
@@ -425,12 +441,14 @@ int bonsai_forces(bonsai_ctx *ctx, float theta, float eps, float *acc, float *po
         return fail(ctx, BONSAI_ERR_NOT_READY, "bonsai_forces: call bonsai_build and bonsai_multipoles first");
     c.theta = theta;
     c.eps = eps;
+    const bool ready = c.walk_ready && !caller_captures(c);   // right after the multipoles
     const long long key[] = {c.n, c.arena_gen, c.nsys, c.ncrit, c.group_pack, c.walk_warps, c.list_capacity,
-                             c.max_spin, fbits(theta), fbits(eps), c.block_kmax};
+                             c.max_spin, fbits(theta), fbits(eps), c.block_kmax, ready};
     CK(run_cached(c, c.forces_graph, key, (int)(sizeof key / sizeof key[0]), [&]() -> cudaError_t {
-        const cudaError_t e = launch_reset(c);
+        const cudaError_t e = ready ? cudaSuccess : launch_reset(c, RESET_WALK);
         return e != cudaSuccess ? e : pipeline_forces(c, theta, eps);
     }));
+    c.walk_ready = false;
     c.have_acc = true;
     if (acc || pot) {
         if (on_device) {
@@ -489,6 +507,7 @@ int bonsai_step(bonsai_ctx *ctx, float dt) {
         c.graph_dt = dt; c.graph_theta = c.theta; c.graph_eps = c.eps; c.graph_n = c.n;
         c.graph_timing = c.stage_timing;
     }
+    c.dom_ready = c.walk_ready = false;
     c.built = c.moments_ready = c.have_acc = c.tree_fresh = true;
     c.timed_step = c.stage_timing;
     return BONSAI_OK;
@@ -537,6 +556,7 @@ int bonsai_autotune(bonsai_ctx *ctx, float theta, float eps, int *best_ncrit, in
             c.walk_warps = w;
             c.list_capacity = caps[wc % 3];
             // one untimed walk, then the mean of two timed ones
+            c.walk_ready = false;
             if ((e = launch_reset(c)) != cudaSuccess || (e = pipeline_forces(c, theta, eps)) != cudaSuccess) break;
             if ((e = cudaEventRecord(e0, c.stream)) != cudaSuccess) break;
             for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {

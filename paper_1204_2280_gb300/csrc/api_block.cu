@@ -180,6 +180,7 @@ static cudaError_t block_cycle(Ctx &c, float dt_max, int kmax, float eta, int re
     const float cc = block_constant(dt_max, eta, c.eps);
     const unsigned nsub = 1u << kmax;
     cudaError_t e;
+    c.walk_ready = c.dom_ready = false;
     c.blk_walked = c.blk_rebuilt = 0;
     k_block_accum<<<1, 32, 0, c.stream>>>(c.st, 1);
     k_block_open<<<grid, 256, 0, c.stream>>>(c.vel4, c.acc4, n, cc, kmax, dtm, c.st);

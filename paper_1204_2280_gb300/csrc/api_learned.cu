@@ -363,6 +363,7 @@ int bonsai_learn_samples(bonsai_ctx *ctx, float theta, float eps, int ntar, unsi
     if (c.step_graph) { cudaGraphExecDestroy(c.step_graph); c.step_graph = nullptr; }
     c.graph_n = -1;
     CCK(cudaMemcpyAsync(tg, pool.data(), sizeof(uint32_t) * ntar, cudaMemcpyHostToDevice, c.stream));
+    c.walk_ready = false;
     CCK(launch_reset(c));
     CCK(launch_walk(c, theta, eps, true));
     CCK(launch_direct(c, tg, ntar, eps, c.judge_partial, JUDGE_SPLIT, c.judge_direct));
@@ -438,6 +439,7 @@ int bonsai_forces_learned(bonsai_ctx *ctx, float eps, float *acc, float *pot, in
     if (!c.moments_ready)
         return cfail(ctx, BONSAI_ERR_NOT_READY, "bonsai_forces_learned: call bonsai_build and bonsai_multipoles first");
     if (!(eps > 0.f)) return cfail(ctx, BONSAI_ERR_INVALID_ARG, "bonsai_forces_learned: eps > 0");
+    c.walk_ready = false;
     CCK(launch_reset(c));
     CCK(pipeline_learned_forces(c, eps));
     c.have_acc = true;

@@ -69,6 +69,10 @@ constexpr long long STAGE_MIN_FLOATS = 4096;           // staging area floor (ge
 constexpr int ENTRY_ROW = NROWS;                       // build: entries per block (a row that is not scanned)
 constexpr int BUILD_ROWS = NROWS + 1;                  // build: per-block count rows
 
+// What launch_reset clears: domain boxes, radix sort counts, walk queues and totals.
+constexpr int RESET_DOMAIN = 1, RESET_SORT = 2, RESET_WALK = 4;
+constexpr int PACK_BLOCKS = 1216;                      // body packing: blocks (eight per SM)
+
 // Device status bits (ORed by kernels, read and cleared by bonsai_sync).
 constexpr unsigned ST_CAPACITY = 1u;
 constexpr unsigned ST_TIMEOUT = 2u;
@@ -98,6 +102,7 @@ struct DevState {
     unsigned long long cyc_inter[2];  // block steps, last cycle: n_pc, n_pp summed over substeps
     unsigned hold_tile;               // testing aid: sort tile hold_tile - 1 never publishes (0: off)
     unsigned blk_next;                // block steps: first substep after the last kick at which a step ends
+    unsigned pack_done;               // body packing: blocks that have finished
     unsigned mom_starts;              // multipoles: internal cells whose children are all leaves
 };
 
@@ -160,12 +165,15 @@ struct Ctx {
     uint2 *counts = nullptr;         // per body (n_pc, n_pp), sorted order
     float *feat = nullptr;           // per body FEAT_STRIDE walk features (learned correction), sorted order
     // staging for host transfers and caller-order outputs
+    float *pack_box = nullptr;       // body packing: the blocks' boxes (6 floats each)
     float *stage = nullptr;          // 7 floats per body, at least STAGE_MIN_FLOATS
     long long stage_floats = 0;      // its size
     DevState *st = nullptr;          // device
     DevState *st_host = nullptr;     // pinned mirror for reads
 
     // pipeline state
+    bool dom_ready = false;          // the domain box of the loaded bodies is on the device (one system, no build yet)
+    bool walk_ready = false;         // the walk queues are reset since the last walk
     bool have_bodies = false, built = false, moments_ready = false, have_acc = false;
     long long arena_limit = 0;       // bytes; 0: no cap on the body arena
     bool tree_fresh = false;         // the tree was built from the current positions (no refit since)
@@ -267,7 +275,7 @@ __device__ __forceinline__ unsigned long long key_prefix(unsigned long long k, i
 }
 
 // ---- launchers (host) ------------------------------------------------------
-cudaError_t launch_reset(Ctx &c);
+cudaError_t launch_reset(Ctx &c, int what = RESET_DOMAIN | RESET_SORT | RESET_WALK);
 cudaError_t launch_domains(Ctx &c);
 cudaError_t launch_fill_sysid(Ctx &c);
 cudaError_t launch_pack(Ctx &c, const float *pos, const float *mass, const float *vel);
@@ -284,7 +292,7 @@ cudaError_t launch_sort(Ctx &c);
 cudaError_t launch_reorder(Ctx &c);
 cudaError_t launch_build(Ctx &c);
 cudaError_t launch_internal_counts(Ctx &c);
-cudaError_t launch_multipoles(Ctx &c);
+cudaError_t launch_multipoles(Ctx &c, bool reset_walk = false);
 cudaError_t launch_multipoles_refit(Ctx &c);
 cudaError_t launch_cell_cubes(Ctx &c);
 cudaError_t launch_sph_walk(Ctx &c, const float *hs, const float4 *cext, float *rho_s, int32_t *cnt_s);

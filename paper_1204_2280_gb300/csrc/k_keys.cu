@@ -10,25 +10,24 @@ namespace bonsai {
 // ---------------------------------------------------------------------------
 __global__ void k_reset(DevState *st, int what, int nsys) {
     int t = threadIdx.x;
-    if (what & 1) {                        // build inputs
+    if (what & RESET_DOMAIN) {
         for (int i = t; i < 3 * nsys; i += blockDim.x) {
             int sys = i / 3, d = i % 3;
             st->dom[6 * sys + d] = 0x7fffffff;
             st->dom[6 * sys + 3 + d] = (int)0x80000000;
         }
+    }
+    if (what & RESET_SORT) {
         for (int i = t; i < (SORT_PASSES + 1) * SORT_RADIX; i += blockDim.x) st->hist[i] = 0;
         if (t < SORT_PASSES + 1) st->sort_tile[t] = 0;
     }
-    if (what & 2) {                        // walk inputs
+    if (what & RESET_WALK) {
         if (t == 0) { st->walk_next = 0; st->walk_next2 = 0; st->inter[0] = 0; st->inter[1] = 0; }
-    }
-    if (what & 4) {
-        if (t < 8) st->diag[t] = 0.0;
     }
 }
 
-cudaError_t launch_reset(Ctx &c) {
-    k_reset<<<1, 256, 0, c.stream>>>(c.st, 7, c.nsys);
+cudaError_t launch_reset(Ctx &c, int what) {
+    k_reset<<<1, 256, 0, c.stream>>>(c.st, what, c.nsys);
     return cudaGetLastError();
 }
 
@@ -52,25 +51,94 @@ cudaError_t launch_fill_sysid(Ctx &c) {
 
 // ---------------------------------------------------------------------------
 // Caller arrays (pos N x 3, mass N, vel N x 3 or null) -> pos4_alt, vel4_alt,
-// id_alt = caller index.  Flags non-finite input.
-__global__ void k_pack(const float *__restrict__ pos, const float *__restrict__ mass,
-                       const float *__restrict__ vel, int n, float4 *pos4,
-                       float4 *vel4, uint32_t *id, DevState *st) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2], m = mass[i];
-    float vx = 0.f, vy = 0.f, vz = 0.f;
-    if (vel) { vx = vel[3 * i]; vy = vel[3 * i + 1]; vz = vel[3 * i + 2]; }
-    if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(m))) atomicOr(&st->status, ST_NAN);
-    pos4[i] = make_float4(x, y, z, m);
-    vel4[i] = make_float4(vx, vy, vz, 0.f);
-    id[i] = (uint32_t)i;
+// id_alt = caller index, one system (sysid 0, its offsets), and the domain
+// box of all positions for the first build: each block's box goes to `part`,
+// the last block to finish adds them up (the separate pass over the bodies,
+// with a reset before it and two small copies here, cost five operations of 2
+// to 4 us each at small sizes and 20 us of reading at 2^20).  Flags
+// non-finite input.
+__device__ __forceinline__ void warp_box(float (&v)[6]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            v[d] = fminf(v[d], __shfl_xor_sync(0xffffffffu, v[d], o));
+            v[3 + d] = fmaxf(v[3 + d], __shfl_xor_sync(0xffffffffu, v[3 + d], o));
+        }
+}
+
+constexpr int PACK_BODIES_THREADS = 256;
+
+__global__ void __launch_bounds__(PACK_BODIES_THREADS)
+k_pack(const float *__restrict__ pos, const float *__restrict__ mass, const float *__restrict__ vel, int n,
+       float4 *pos4, float4 *vel4, uint32_t *id, uint8_t *sysid, float *part, DevState *st) {
+    constexpr int NW = PACK_BODIES_THREADS / 32;
+    __shared__ float red[6][NW];
+    __shared__ bool s_last;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    bool bad = false;
+    for (long long i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const float x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2], m = mass[i];
+        float vx = 0.f, vy = 0.f, vz = 0.f;
+        if (vel) { vx = vel[3 * i]; vy = vel[3 * i + 1]; vz = vel[3 * i + 2]; }
+        bad |= !(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(m));
+        pos4[i] = make_float4(x, y, z, m);
+        vel4[i] = make_float4(vx, vy, vz, 0.f);
+        id[i] = (uint32_t)i;
+        sysid[i] = 0;
+        v[0] = fminf(v[0], x); v[1] = fminf(v[1], y); v[2] = fminf(v[2], z);
+        v[3] = fmaxf(v[3], x); v[4] = fmaxf(v[4], y); v[5] = fmaxf(v[5], z);
+    }
+    if (__any_sync(0xffffffffu, bad) && l == 0) atomicOr(&st->status, ST_NAN);
+    warp_box(v);
+    if (l == 0)
+#pragma unroll
+        for (int d = 0; d < 6; d++) red[d][w] = v[d];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        float r = red[threadIdx.x][0];
+        for (int k = 1; k < NW; k++)
+            r = threadIdx.x < 3 ? fminf(r, red[threadIdx.x][k]) : fmaxf(r, red[threadIdx.x][k]);
+        part[6 * blockIdx.x + threadIdx.x] = r;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&st->pack_done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+#pragma unroll
+    for (int d = 0; d < 6; d++) v[d] = d < 3 ? INFINITY : -INFINITY;
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x)
+#pragma unroll
+        for (int d = 0; d < 6; d++) {
+            const float q = __ldcg(part + 6 * k + d);
+            v[d] = d < 3 ? fminf(v[d], q) : fmaxf(v[d], q);
+        }
+    warp_box(v);
+    if (l == 0)
+#pragma unroll
+        for (int d = 0; d < 6; d++) red[d][w] = v[d];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        float r = red[threadIdx.x][0];
+        for (int k = 1; k < NW; k++)
+            r = threadIdx.x < 3 ? fminf(r, red[threadIdx.x][k]) : fmaxf(r, red[threadIdx.x][k]);
+        st->dom[threadIdx.x] = f2ord(r);
+    }
+    if (threadIdx.x == 0) {
+        st->pack_done = 0u;
+        st->sys_off[0] = 0u;
+        st->sys_off[1] = (unsigned)n;
+    }
 }
 
 cudaError_t launch_pack(Ctx &c, const float *pos, const float *mass, const float *vel) {
-    int n = (int)c.n;
-    k_pack<<<(n + 255) / 256, 256, 0, c.stream>>>(pos, mass, vel, n, c.pos4_alt, c.vel4_alt,
-                                                  c.id_alt, c.st);
+    const int n = (int)c.n;
+    const int grid = min((n + PACK_BODIES_THREADS - 1) / PACK_BODIES_THREADS, PACK_BLOCKS);
+    k_pack<<<grid, PACK_BODIES_THREADS, 0, c.stream>>>(pos, mass, vel, n, c.pos4_alt, c.vel4_alt, c.id_alt, c.sysid,
+                                                       c.pack_box, c.st);
     return cudaGetLastError();
 }
 

@@ -139,6 +139,7 @@ __device__ __forceinline__ void cp_async16(float4 *sdst, const float4 *gsrc, boo
 
 struct MomArrays {
     const DevState *__restrict__ stc;
+    DevState *st;                     // not NULL: reset the walk's queues and totals
     const uint2 *__restrict__ cell_body;
     const uint2 *__restrict__ cell_link;
     const uint8_t *__restrict__ cell_level;
@@ -349,6 +350,10 @@ __device__ __forceinline__ void combine_cell(unsigned c, int lv, uint2 plk, unsi
 template <bool REFIT>
 __global__ void __launch_bounds__(256, MOM_MINB)
 k_mom_leaves(MomArrays a) {
+    if (a.st && blockIdx.x == 0 && threadIdx.x == 0) {   // the walk that follows starts from empty queues
+        a.st->walk_next = 0u; a.st->walk_next2 = 0u;
+        a.st->inter[0] = 0ull; a.st->inter[1] = 0ull;
+    }
     const unsigned nc = a.stc->ncells;
     if (a.stc->status & ST_TIMEOUT) return;
     const unsigned lane = threadIdx.x & 31u;
@@ -437,8 +442,8 @@ static unsigned multipole_blocks(const Ctx &c) {
     return (unsigned)((cells + 255) / 256);
 }
 
-static MomArrays mom_arrays(Ctx &c, bool refit) {
-    return MomArrays{c.st, c.cell_body, c.cell_link, c.cell_level, c.cell_parent, c.cell_done, c.pos4, c.keys,
+static MomArrays mom_arrays(Ctx &c, bool refit, bool reset) {
+    return MomArrays{c.st, reset ? c.st : nullptr, c.cell_body, c.cell_link, c.cell_level, c.cell_parent, c.cell_done, c.pos4, c.keys,
                      c.sysid, c.mono, c.quadA, c.quadB, c.delta, c.shadow, refit ? c.cext : nullptr, c.nsys > 1,
                      c.cell_start, &c.st->mom_starts};
 }
@@ -453,12 +458,14 @@ static cudaError_t launch_mom(Ctx &c, const MomArrays &a) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_multipoles(Ctx &c) { return launch_mom<false>(c, mom_arrays(c, false)); }
+cudaError_t launch_multipoles(Ctx &c, bool reset_walk) {
+    return launch_mom<false>(c, mom_arrays(c, false, reset_walk));
+}
 
 // Moments of the existing cells at the bodies' current positions (block time
 // steps between rebuilds), with each cell's cube enlarged to hold its bodies.
 cudaError_t launch_multipoles_refit(Ctx &c) {
-    return launch_mom<true>(c, mom_arrays(c, true));
+    return launch_mom<true>(c, mom_arrays(c, true, false));
 }
 
 // cext[c] = (geometric centre, l / 2) of every cell from its first body's

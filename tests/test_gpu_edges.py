@@ -188,3 +188,40 @@ def test_judge_sizes(n):
     e = np.where(norm > 0, np.linalg.norm(acc[ids] - a, axis=1) / np.maximum(norm, 1e-300), 0.0)
     ref = np.percentile(e, 99)
     assert abs(p - ref) <= 1e-4 * ref + 1e-6
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 5000, 1216 * 256 + 1])
+def test_domain_of_loaded_bodies(n):
+    """The domain box that loading leaves for the first build (block boxes,
+    last block adds up), against the oracle, also after other bodies, for two
+    systems, after a rebuild, and with walks repeated without multipoles
+    between them."""
+    import oracle
+    rng = np.random.default_rng(n)
+    acc = [np.zeros((n, 3), np.float32) for _ in range(3)]
+    with B.Bonsai(B.Config(ncrit=32)) as bz:
+        for scale in (1.0, 1e-3, 50.0):
+            pos = (rng.normal(size=(n, 3)) * scale + scale).astype(np.float32)
+            mass = np.full(n, 1.0 / n, np.float32)
+            bz.set_bodies(pos, mass).build()
+            mn, S = oracle.domain(pos)
+            for _ in range(2):
+                m, s = B.bonsai_get_domain(bz.ctx)
+                assert np.array_equal(m, mn) and s == S
+                bz.build()
+        bz.multipoles().forces(0.75, 0.1, acc[0])
+        tot = B.bonsai_get_counts(bz.ctx)[2]
+        bz.forces(0.75, 0.1, acc[1])                 # no multipoles between: the queues start over
+        assert B.bonsai_get_counts(bz.ctx)[2] == tot
+        bz.multipoles()
+        assert B.bonsai_get_counts(bz.ctx)[2] == tot  # the last walk's totals stay readable
+        bz.forces(0.75, 0.1, acc[2])
+        assert B.bonsai_get_counts(bz.ctx)[2] == tot
+        assert np.array_equal(acc[0], acc[1]) and np.array_equal(acc[0], acc[2])
+        if n > 1:
+            bz.set_bodies(pos, mass).set_systems([0, n // 2, n]).build()
+            m, s = B.bonsai_get_domains(bz.ctx, 2)
+            for k, (lo, hi) in enumerate(((0, n // 2), (n // 2, n))):
+                mn, S = oracle.domain(pos[lo:hi])
+                assert np.array_equal(m[k], mn) and s[k] == S
+        bz.sync()
