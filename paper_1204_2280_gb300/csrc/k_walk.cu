@@ -320,7 +320,7 @@ __device__ __forceinline__ void walk_pop(const unsigned *stk, int &sp, int lane,
 #define WALK_MIN_BLOCKS2 0
 #endif
 #ifndef WALK_SMALL_LAST
-#define WALK_SMALL_LAST 16          // > 0: groups of at most this many bodies in a second pass
+#define WALK_SMALL_LAST 16          // groups of at most this many bodies in a second pass
 #endif
 #ifndef WALK_MAXNREG1
 #define WALK_MAXNREG1 0             // > 0: register cap of the one-body-per-lane walk
@@ -330,7 +330,10 @@ __device__ __forceinline__ void walk_pop(const unsigned *stk, int &sp, int lane,
 #else
 #define WALK_ATTRS __launch_bounds__(256, BPL == 1 ? WALK_MIN_BLOCKS1 : BPL == 2 ? WALK_MIN_BLOCKS2 : 2)
 #endif
-template <int BPL, bool FEAT, bool BLOCK>
+// SPLIT (one body per lane): groups of 33..64 bodies are two items of up to
+// 32, walked by two warps with the whole group's box; each body gets the same
+// operations in the same order as from one warp with two bodies per lane.
+template <int BPL, bool FEAT, bool BLOCK, bool SPLIT>
 __global__ void WALK_ATTRS
 k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__ groups,
        const float4 *__restrict__ pos4, const float2 *__restrict__ delta, float inv_theta,
@@ -359,28 +362,33 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
         unsigned g = 0;
         if (lane == 0) g = atomicAdd(queue, 1u);
         g = __shfl_sync(0xffffffffu, g, 0);
-#if WALK_SMALL_LAST
-        // two passes over the groups: larger ones first, then those of at
-        // most WALK_SMALL_LAST bodies (a shorter tail at the end of the walk)
-        const bool second = g >= ngroups;
-        if (second) g -= ngroups;
-#endif
+        // two passes over the groups: larger ones first (SPLIT: two tickets
+        // each), then those of at most WALK_SMALL_LAST bodies (a shorter tail
+        // at the end of the walk)
+        const unsigned first = SPLIT ? 2u * ngroups : ngroups;
+        const bool second = g >= first;
+        int half = 0;
+        if (second) {
+            g -= first;
+        } else if (SPLIT) {
+            half = (int)(g & 1u);
+            g >>= 1;
+        }
         if (g >= ngroups) break;
         const uint2 gr = groups[g];
         const int gb = (int)gr.x, ng = (int)gr.y;
         // groups this instantiation can never take (by size; without block
         // time steps every body takes part, so the size decides)
-        if (!BLOCK && walk_bpl(ng, three) != BPL) continue;
+        if (!BLOCK && !SPLIT && walk_bpl(ng, three) != BPL) continue;
+        if (SPLIT && half && ng <= 32) continue;
         if (BLOCK && ((BPL == 2 && walk_bpl(ng, three) != 2) || (BPL == 3 && ng <= 16))) continue;
-#if WALK_SMALL_LAST
         if (second != (ng <= WALK_SMALL_LAST)) continue;
-#endif
         // Body slots and source phases.
         // Block time steps, groups of <= 32 bodies: the active bodies are
         // compacted into the first body slots (in body order), and the
         // instantiation and slot count follow the active count (all active:
         // the plain layout, so the same sums as a plain walk).
-        int nslot = ng;
+        int nslot = SPLIT ? min(32, ng - 32 * half) : ng;
         bool act = false;
         unsigned am = 0u;
         if (BLOCK && ng <= 32) {
@@ -394,7 +402,7 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
             if (act) R.leaf[__popc(am & lt)].x = (unsigned)lane;
             __syncwarp();
         }
-        const int lg = walk_lg<BPL>(nslot);
+        const int lg = SPLIT && ng > 32 ? 5 : walk_lg<BPL>(nslot);
         const int slots = 1 << lg;
         const int bslot = lane & (slots - 1), phase = lane >> lg;
         bool live[BPL];
@@ -413,8 +421,14 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
                 // only the bodies whose step ends at this substep
                 live[b] = block_active(actv[gb + slot].w, act_s, act_kmax);
             }
+            if (SPLIT) body += 32 * half;
             bi[b] = gb + (live[b] ? body : 0);
             me[b] = pos4[bi[b]];
+            if (SPLIT && lane + 32 * (1 - half) < ng && ng > 32) {   // the other half's bodies widen the box
+                const float4 o = pos4[gb + lane + 32 * (1 - half)];
+                bx0 = fminf(bx0, o.x); by0 = fminf(by0, o.y); bz0 = fminf(bz0, o.z);
+                bx1 = fmaxf(bx1, o.x); by1 = fmaxf(by1, o.y); bz1 = fmaxf(bz1, o.z);
+            }
             if (live[b]) {
                 bx0 = fminf(bx0, me[b].x); by0 = fminf(by0, me[b].y); bz0 = fminf(bz0, me[b].z);
                 bx1 = fmaxf(bx1, me[b].x); by1 = fmaxf(by1, me[b].y); bz1 = fmaxf(bz1, me[b].z);
@@ -430,7 +444,7 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
             bz1 = fmaxf(bz1, __shfl_xor_sync(0xffffffffu, bz1, o));
         }
         // Live body slots (bit = slot); a group without one is skipped.
-        unsigned nlive = (unsigned)ng;
+        unsigned nlive = (unsigned)nslot;
         if (BLOCK) {                               // a group without a live body is skipped
             nlive = 0u;
 #pragma unroll
@@ -609,7 +623,7 @@ size_t walk_smem_bytes(int warps, int stack_cap) {
 
 // Function attribute and occupancy are set up once per shape, before any
 // stream capture of a step (the first step always runs eagerly).
-template <int BPL, bool FEAT, bool BLOCK>
+template <int BPL, bool FEAT, bool BLOCK, bool SPLIT = false>
 static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned *gate, bool three, cudaStream_t stream) {
     const unsigned polls = (unsigned)(c.max_spin < 0xffffffffll ? c.max_spin : 0xffffffffll);
     const int warps = c.walk_warps;
@@ -618,22 +632,34 @@ static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned 
     // that device's
     static size_t attr_done[MAX_DEVICES] = {}, occ_smem[MAX_DEVICES] = {};
     static int occ_warps[MAX_DEVICES] = {}, occ_per_sm[MAX_DEVICES] = {};
-    cudaError_t ea = allow_dyn_smem((const void *)k_walk<BPL, FEAT, BLOCK>, smem, attr_done);
+    cudaError_t ea = allow_dyn_smem((const void *)k_walk<BPL, FEAT, BLOCK, SPLIT>, smem, attr_done);
     if (ea != cudaSuccess) return ea;
     const int dv = c.device;
     if (dv < 0 || dv >= MAX_DEVICES) return cudaErrorInvalidDevice;
     if (occ_warps[dv] != warps || occ_smem[dv] != smem) {
         int per = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<BPL, FEAT, BLOCK>, warps * 32, smem);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<BPL, FEAT, BLOCK, SPLIT>, warps * 32, smem);
         if (e != cudaSuccess) return e;
         occ_warps[dv] = warps; occ_smem[dv] = smem; occ_per_sm[dv] = per < 1 ? 1 : per;
     }
-    k_walk<BPL, FEAT, BLOCK><<<c.num_sms * occ_per_sm[dv], warps * 32, smem, stream>>>(
+    k_walk<BPL, FEAT, BLOCK, SPLIT><<<c.num_sms * occ_per_sm[dv], warps * 32, smem, stream>>>(
         c.st, c.st, c.groups, c.pos4, c.delta, 1.0f / theta, c.cell_link, c.mono, c.quadA, c.quadB, c.sysid, eps,
         c.list_capacity, polls, c.acc4, c.counts, c.cell_level, c.feat, gate,
         BLOCK ? c.vel4 : nullptr, c.block_s, c.block_kmax, three);
     return cudaGetLastError();
 }
+
+// Up to this many bodies the groups of 33..64 are two items of one body per
+// lane instead of one with two.  Each item traverses the tree, but a group's
+// chain of tiles is half as long, the kernel has 24 warps per SM instead of
+// 12 and no second launch follows: with few groups per warp the longest chain
+// decides.  Evaluations, two bodies per lane / split, ncrit 64: 74 / 68 us at
+// 2^12, 112 / 92 at 2^14, 209 / 191 at 2^16, 592 / 591 at 2^18 and 2251 / 2280
+// at 2^20, where the doubled traversals cost more (theta 0.5, 200,003 bodies:
+// 1253 / 1142).
+#ifndef WALK_SPLIT_MAX_N
+#define WALK_SPLIT_MAX_N (1 << 18)
+#endif
 
 // One persistent launch per instantiation that can receive groups (group
 // sizes are at most ncrit; oversize leaves are cut into chunks of ncrit).
@@ -661,6 +687,9 @@ cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features, const uns
                         : launch_walk_t<1, false, false>(c, theta, eps, gate, three, st);
     };
     const int second = c.ncrit >= WALK_BPL2_FROM ? 2 : three ? 3 : 0;
+    if (second == 2 && c.block_kmax < 0 && c.n <= WALK_SPLIT_MAX_N)
+        return features ? launch_walk_t<1, true, false, true>(c, theta, eps, gate, false, c.stream)
+                        : launch_walk_t<1, false, false, true>(c, theta, eps, gate, false, c.stream);
     if (second == 0) return one(1, c.stream);
     cudaError_t e = cudaEventRecord(c.ev_fork, c.stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c.side, c.ev_fork, 0);

@@ -225,3 +225,51 @@ def test_domain_of_loaded_bodies(n):
                 mn, S = oracle.domain(pos[lo:hi])
                 assert np.array_equal(m[k], mn) and s[k] == S
         bz.sync()
+
+
+@pytest.mark.parametrize("ncrit,pack,n", [(64, 0, 1), (64, 0, 33), (64, 0, 65), (33, 0, 500), (64, 1, 3000),
+                                          (64, 0, 12000), (48, 1, 20000), (64, 1, (1 << 18) - 3)])
+def test_split_groups_equal_two_bodies_per_lane(ncrit, pack, n):
+    """Groups of 33..64 bodies walked as two items (up to 2^18 bodies)
+    against block time steps' walk, which has two bodies per lane: a one-level
+    cycle moves every body as the step does, bit for bit, with the same
+    interaction counts.  Identical positions, oversize leaves and single
+    bodies included; and the forces of a system alone against those beside
+    a system large enough for two bodies per lane."""
+    import torch
+    from gpu_common import edge_bodies
+    b = edge_bodies(n, 5) if n > 200 else None
+    rng = np.random.default_rng(n)
+    pos = b.pos if b else rng.normal(size=(n, 3)).astype(np.float32)
+    mass = b.mass if b else np.full(n, 1.0 / n, np.float32)
+    mass = mass.astype(np.float32)
+    out = []
+    for block in (False, True):
+        with B.Bonsai(B.Config(ncrit=ncrit, group_pack=pack)) as bz:
+            bz.set_bodies(pos, mass).build().multipoles().forces(0.9, 0.01)
+            if block:
+                bz.block_cycle(1.0 / 64, 0, 0.2)
+            else:
+                bz.step(1.0 / 64)
+            x, v = np.zeros((n, 3), np.float32), np.zeros((n, 3), np.float32)
+            B.bonsai_get_bodies(bz.ctx, x, v)
+            bz.sync()
+            out.append((x, v, B.bonsai_get_counts(bz.ctx)))
+    (x0, v0, c0), (x1, v1, c1) = out
+    assert np.array_equal(x0, x1) and np.array_equal(v0, v1)
+    assert np.array_equal(c0[0], c1[0]) and np.array_equal(c0[1], c1[1]) and c0[2] == c1[2]
+    # the forces themselves: alone, and beside a larger system
+    m = 1 << 18
+    pos2 = np.concatenate([pos, rng.normal(size=(m, 3)).astype(np.float32)])
+    mass2 = np.concatenate([mass, np.full(m, 1.0 / m, np.float32)])
+    res = []
+    for p, q, off in ((pos, mass, None), (pos2, mass2, [0, n, n + m])):
+        with B.Bonsai(B.Config(ncrit=ncrit, group_pack=pack)) as bz:
+            acc, pot = torch.zeros(len(q), 3, device="cuda"), torch.zeros(len(q), device="cuda")
+            bz.set_bodies(p, q)
+            if off:
+                bz.set_systems(off)
+            bz.build().multipoles().forces(0.9, 0.01, acc, pot)
+            bz.sync()
+            res.append((acc[:n].cpu().numpy(), pot[:n].cpu().numpy()))
+    assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])
