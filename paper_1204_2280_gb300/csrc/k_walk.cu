@@ -330,10 +330,12 @@ __device__ __forceinline__ void walk_pop(const unsigned *stk, int &sp, int lane,
 #else
 #define WALK_ATTRS __launch_bounds__(256, BPL == 1 ? WALK_MIN_BLOCKS1 : BPL == 2 ? WALK_MIN_BLOCKS2 : 2)
 #endif
-// SPLIT (one body per lane): groups of 33..64 bodies are two items of up to
-// 32, walked by two warps with the whole group's box; each body gets the same
-// operations in the same order as from one warp with two bodies per lane.
-template <int BPL, bool FEAT, bool BLOCK, bool SPLIT>
+// SPLIT (one body per lane): the groups that a second instantiation would
+// take are walked in SPLIT parts by as many warps, each with the whole group's
+// box: 2 parts of up to 32 bodies (groups of 33..64) or 3 of up to 8 (groups
+// of 17..24, four phases).  Each body gets the same operations in the same
+// order as from one warp with two or three bodies per lane.
+template <int BPL, bool FEAT, bool BLOCK, int SPLIT>
 __global__ void WALK_ATTRS
 k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__ groups,
        const float4 *__restrict__ pos4, const float2 *__restrict__ delta, float inv_theta,
@@ -355,6 +357,7 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
         ((stc->status & ST_TIMEOUT) || (gate && *gate == 0u) || stc->ncells == 0u) ? 0u : stc->ngroups;
     const float eps2 = eps * eps;
     const float2 eps2x2 = make_float2(eps2, eps2);
+    constexpr int part_size = SPLIT == 2 ? 32 : 8;
     const unsigned lt = lanemask_lt_w();
     unsigned *queue = BPL == 1 ? &st->walk_next : &st->walk_next2;
 
@@ -362,17 +365,17 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
         unsigned g = 0;
         if (lane == 0) g = atomicAdd(queue, 1u);
         g = __shfl_sync(0xffffffffu, g, 0);
-        // two passes over the groups: larger ones first (SPLIT: two tickets
-        // each), then those of at most WALK_SMALL_LAST bodies (a shorter tail
+        // two passes over the groups: larger ones first (SPLIT: a ticket per
+        // part), then those of at most WALK_SMALL_LAST bodies (a shorter tail
         // at the end of the walk)
-        const unsigned first = SPLIT ? 2u * ngroups : ngroups;
+        const unsigned first = SPLIT ? (unsigned)SPLIT * ngroups : ngroups;
         const bool second = g >= first;
-        int half = 0;
+        int part = 0;
         if (second) {
             g -= first;
         } else if (SPLIT) {
-            half = (int)(g & 1u);
-            g >>= 1;
+            part = (int)(g % (unsigned)(SPLIT ? SPLIT : 1));
+            g /= (unsigned)(SPLIT ? SPLIT : 1);
         }
         if (g >= ngroups) break;
         const uint2 gr = groups[g];
@@ -380,7 +383,8 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
         // groups this instantiation can never take (by size; without block
         // time steps every body takes part, so the size decides)
         if (!BLOCK && !SPLIT && walk_bpl(ng, three) != BPL) continue;
-        if (SPLIT && half && ng <= 32) continue;
+        const bool cut = SPLIT == 2 ? ng > 32 : SPLIT == 3 ? ng > 16 && ng <= 24 : false;   // walked in parts
+        if (SPLIT && part && (!cut || part_size * part >= ng)) continue;
         if (BLOCK && ((BPL == 2 && walk_bpl(ng, three) != 2) || (BPL == 3 && ng <= 16))) continue;
         if (second != (ng <= WALK_SMALL_LAST)) continue;
         // Body slots and source phases.
@@ -388,7 +392,7 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
         // compacted into the first body slots (in body order), and the
         // instantiation and slot count follow the active count (all active:
         // the plain layout, so the same sums as a plain walk).
-        int nslot = SPLIT ? min(32, ng - 32 * half) : ng;
+        int nslot = cut ? min(part_size, ng - part_size * part) : ng;
         bool act = false;
         unsigned am = 0u;
         if (BLOCK && ng <= 32) {
@@ -402,7 +406,7 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
             if (act) R.leaf[__popc(am & lt)].x = (unsigned)lane;
             __syncwarp();
         }
-        const int lg = SPLIT && ng > 32 ? 5 : walk_lg<BPL>(nslot);
+        const int lg = cut ? (SPLIT == 2 ? 5 : 3) : walk_lg<BPL>(nslot);
         const int slots = 1 << lg;
         const int bslot = lane & (slots - 1), phase = lane >> lg;
         bool live[BPL];
@@ -421,13 +425,16 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
                 // only the bodies whose step ends at this substep
                 live[b] = block_active(actv[gb + slot].w, act_s, act_kmax);
             }
-            if (SPLIT) body += 32 * half;
+            if (SPLIT) body += part_size * part;
             bi[b] = gb + (live[b] ? body : 0);
             me[b] = pos4[bi[b]];
-            if (SPLIT && lane + 32 * (1 - half) < ng && ng > 32) {   // the other half's bodies widen the box
-                const float4 o = pos4[gb + lane + 32 * (1 - half)];
-                bx0 = fminf(bx0, o.x); by0 = fminf(by0, o.y); bz0 = fminf(bz0, o.z);
-                bx1 = fmaxf(bx1, o.x); by1 = fmaxf(by1, o.y); bz1 = fmaxf(bz1, o.z);
+            if (SPLIT && cut) {                        // the other parts' bodies widen the box
+                const int other = SPLIT == 2 ? lane + 32 * (1 - part) : lane;
+                if (other < ng) {
+                    const float4 o = pos4[gb + other];
+                    bx0 = fminf(bx0, o.x); by0 = fminf(by0, o.y); bz0 = fminf(bz0, o.z);
+                    bx1 = fmaxf(bx1, o.x); by1 = fmaxf(by1, o.y); bz1 = fmaxf(bz1, o.z);
+                }
             }
             if (live[b]) {
                 bx0 = fminf(bx0, me[b].x); by0 = fminf(by0, me[b].y); bz0 = fminf(bz0, me[b].z);
@@ -623,7 +630,7 @@ size_t walk_smem_bytes(int warps, int stack_cap) {
 
 // Function attribute and occupancy are set up once per shape, before any
 // stream capture of a step (the first step always runs eagerly).
-template <int BPL, bool FEAT, bool BLOCK, bool SPLIT = false>
+template <int BPL, bool FEAT, bool BLOCK, int SPLIT = 0>
 static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned *gate, bool three, cudaStream_t stream) {
     const unsigned polls = (unsigned)(c.max_spin < 0xffffffffll ? c.max_spin : 0xffffffffll);
     const int warps = c.walk_warps;
@@ -649,14 +656,18 @@ static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned 
     return cudaGetLastError();
 }
 
-// Up to this many bodies the groups of 33..64 are two items of one body per
-// lane instead of one with two.  Each item traverses the tree, but a group's
-// chain of tiles is half as long, the kernel has 24 warps per SM instead of
-// 12 and no second launch follows: with few groups per warp the longest chain
-// decides.  Evaluations, two bodies per lane / split, ncrit 64: 74 / 68 us at
-// 2^12, 112 / 92 at 2^14, 209 / 191 at 2^16, 592 / 591 at 2^18 and 2251 / 2280
-// at 2^20, where the doubled traversals cost more (theta 0.5, 200,003 bodies:
-// 1253 / 1142).
+// Up to these many bodies the groups of a second instantiation are walked in
+// parts by the first.  Each part traverses the tree, but a group's chain of
+// tiles is shorter, the kernel has 24 warps per SM instead of 12 or 16 and no
+// second launch follows: with few groups per warp the longest chain decides.
+// Evaluations, two launches / parts: groups of 33..64 (ncrit 64) 74 / 68 us at
+// 2^12, 112 / 92 at 2^14, 209 / 191 at 2^16, 592 / 591 at 2^18, 2251 / 2280 at
+// 2^20 (theta 0.5, 200,003 bodies: 1253 / 1142); groups of 17..24 (ncrit 32,
+// packed) 79 / 72 at 2^12, 125 / 120 at 2^15, 194 / 191 at 2^16, 300 / 320 at
+// 2^17.  Beyond, the repeated traversals cost more.
+#ifndef WALK_SPLIT3_MAX_N
+#define WALK_SPLIT3_MAX_N (1 << 16)
+#endif
 #ifndef WALK_SPLIT_MAX_N
 #define WALK_SPLIT_MAX_N (1 << 18)
 #endif
@@ -688,8 +699,10 @@ cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features, const uns
     };
     const int second = c.ncrit >= WALK_BPL2_FROM ? 2 : three ? 3 : 0;
     if (second == 2 && c.block_kmax < 0 && c.n <= WALK_SPLIT_MAX_N)
-        return features ? launch_walk_t<1, true, false, true>(c, theta, eps, gate, false, c.stream)
-                        : launch_walk_t<1, false, false, true>(c, theta, eps, gate, false, c.stream);
+        return features ? launch_walk_t<1, true, false, 2>(c, theta, eps, gate, false, c.stream)
+                        : launch_walk_t<1, false, false, 2>(c, theta, eps, gate, false, c.stream);
+    if (second == 3 && c.block_kmax < 0 && c.n <= WALK_SPLIT3_MAX_N)
+        return launch_walk_t<1, false, false, 3>(c, theta, eps, gate, true, c.stream);
     if (second == 0) return one(1, c.stream);
     cudaError_t e = cudaEventRecord(c.ev_fork, c.stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c.side, c.ev_fork, 0);

@@ -228,14 +228,16 @@ def test_domain_of_loaded_bodies(n):
 
 
 @pytest.mark.parametrize("ncrit,pack,n", [(64, 0, 1), (64, 0, 33), (64, 0, 65), (33, 0, 500), (64, 1, 3000),
-                                          (64, 0, 12000), (48, 1, 20000), (64, 1, (1 << 18) - 3)])
-def test_split_groups_equal_two_bodies_per_lane(ncrit, pack, n):
-    """Groups of 33..64 bodies walked as two items (up to 2^18 bodies)
-    against block time steps' walk, which has two bodies per lane: a one-level
+                                          (64, 0, 12000), (48, 1, 20000), (64, 1, (1 << 18) - 3), (32, 1, 17),
+                                          (32, 0, 500), (32, 1, 24), (32, 1, 9000), (24, 1, 30000), (32, 1, 65536)])
+def test_walk_in_parts(ncrit, pack, n):
+    """Groups of 33..64 bodies walked in two parts (up to 2^18 bodies) and of
+    17..24 in three (up to 2^16), against block time steps' walk, which has
+    two or three bodies per lane: a one-level
     cycle moves every body as the step does, bit for bit, with the same
     interaction counts.  Identical positions, oversize leaves and single
     bodies included; and the forces of a system alone against those beside
-    a system large enough for two bodies per lane."""
+    a system large enough for that walk."""
     import torch
     from gpu_common import edge_bodies
     b = edge_bodies(n, 5) if n > 200 else None
