@@ -154,7 +154,6 @@ struct Ctx {
     float2 *quadB = nullptr;
     float2 *delta = nullptr;         // per cell: (|com - centre|, side l; after a refit 2 ext)
     float4 *cext = nullptr;          // per cell after a refit: build-time centre, half side ext holding its bodies
-    double *shadow = nullptr;        // FP64 moments of the top levels (10 per cell)
     uint2 *groups = nullptr;
     // sibling packing (group_pack = 1): the unpacked groups, their cell level
     // (0xff: a run of an oversize leaf), packed-group start flags, and the

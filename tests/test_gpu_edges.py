@@ -275,3 +275,35 @@ def test_walk_in_parts(ncrit, pack, n):
             bz.sync()
             res.append((acc[:n].cpu().numpy(), pot[:n].cpu().numpy()))
     assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])
+
+
+@pytest.mark.parametrize("sizes", [[1], [17], [130], [20000], [30] * 256, [100] * 256, [1, 17, 9000, 16, 600, 2] * 3,
+                                   [17] * 255 + [40000]], ids=lambda s: f"{len(s)}x{s[0]}..{s[-1]}")
+def test_root_moments(sizes):
+    """The roots that a warp combines (none, one or many to a warp) against
+    FP64 sums over each system's bodies: sums of at most a hundred FP32 terms
+    per level of the few levels, errors mostly cancelling, so within 128
+    roundings of the mass, of the extent and of mass times extent^2; and
+    every system's root bit for bit that of the system alone."""
+    rng = np.random.default_rng(len(sizes) + sizes[-1])
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    pos = (rng.normal(size=(off[-1], 3)) + 3.0).astype(np.float32)
+    mass = rng.uniform(0.5, 1.5, off[-1]).astype(np.float32)
+    mass[off[:-1][::3]] = 0.0                            # a system of one massless body too
+    with B.Bonsai(B.Config()) as bz:
+        bz.set_bodies(pos, mass).set_systems(off).build().multipoles()
+        mono, quad = B.bonsai_get_moments(bz.ctx)
+        bz.sync()
+    for k in list(range(0, len(sizes), max(1, len(sizes) // 8))) + [len(sizes) - 1]:
+        p, m = pos[off[k]:off[k + 1]].astype(np.float64), mass[off[k]:off[k + 1]].astype(np.float64)
+        if m.sum() > 0:
+            tol, M, com = 128 * 2.0 ** -24, m.sum(), (m[:, None] * p).sum(0) / m.sum()
+            y, size = p - com, np.abs(p).max()
+            q = np.einsum("i,ij,ik->jk", m, y, y) * 3 - np.eye(3) * (m * (y * y).sum(1)).sum()
+            assert abs(mono[k, 3] - M) <= tol * M
+            assert np.abs(mono[k, :3] - com).max() <= tol * size
+            assert np.abs(quad[k] - q[[0, 1, 2, 0, 0, 1], [0, 1, 2, 1, 2, 2]]).max() <= tol * M * size ** 2
+        with B.Bonsai(B.Config()) as bz:
+            bz.set_bodies(pos[off[k]:off[k + 1]], mass[off[k]:off[k + 1]]).build().multipoles()
+            m1, q1 = B.bonsai_get_moments(bz.ctx)
+        assert np.array_equal(mono[k], m1[0]) and np.array_equal(quad[k], q1[0])
