@@ -360,6 +360,11 @@ k_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restrict__
     constexpr int part_size = SPLIT == 2 ? 32 : 8;
     const unsigned lt = lanemask_lt_w();
     unsigned *queue = BPL == 1 ? &st->walk_next : &st->walk_next2;
+    // Fewer items than warps: only as many warps of each block as there are
+    // items for, so that the blocks that start first do not take them all,
+    // eight to a block, while other SMs idle.  Walks of 8,192 bodies 83 -> 76
+    // us; evaluations of 4,096 bodies 63.7 -> 61.5 us.
+    if ((unsigned)warp * gridDim.x >= (SPLIT ? (unsigned)SPLIT * ngroups : ngroups)) return;
 
     while (true) {
         unsigned g = 0;
