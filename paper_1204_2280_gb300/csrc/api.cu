@@ -65,7 +65,8 @@ void free_bodies(Ctx &c) {
 cudaError_t alloc_bodies(Ctx &c, long long n) {
     free_bodies(c);
     const long long ntiles = (n + SORT_TILE - 1) / SORT_TILE;
-    const long long nbb = (n + BUILD_BODIES - 1) / BUILD_BODIES;
+    // build blocks of any number of bodies up to n
+    const long long nbb = std::max(build_blocks(n), build_blocks(std::min(n, BUILD_SMALL_N)));
     // Cells: at most n leaves and n/(nleaf+1) internal cells per level.
     const long long ccap = n + (long long)MAX_LEVEL * (n / (c.nleaf + 1)) + 64;
     std::vector<std::pair<void **, size_t>> plan;
@@ -77,7 +78,7 @@ cudaError_t alloc_bodies(Ctx &c, long long n) {
     a.take(c.vals, n, plan); a.take(c.vals_alt, n, plan);
     a.take(c.tile_status, (size_t)(SORT_PASSES + 1) * ntiles * SORT_RADIX, plan);
     a.take(c.blockcount, (size_t)BUILD_ROWS * nbb, plan);
-    a.take(c.build_entries, (size_t)nbb * BUILD_BODIES, plan);
+    a.take(c.build_entries, (size_t)build_blocks(n) * build_bodies(n), plan);
     a.take(c.cell_body, ccap, plan); a.take(c.cell_link, ccap, plan);
     a.take(c.cell_level, ccap, plan); a.take(c.cell_parent, ccap, plan);
     a.take(c.cell_done, ccap, plan); a.take(c.cell_cb, ccap, plan); a.take(c.cell_start, ccap, plan);
@@ -99,7 +100,6 @@ cudaError_t alloc_bodies(Ctx &c, long long n) {
     c.arena_gen++;
     c.stage_floats = stage_floats;
     c.ntiles = (int)ntiles;
-    c.nbblocks = (int)nbb;
     c.ccap = ccap;
     c.judge_n = 0;
     return cudaMemsetAsync(base, 0, a.off, c.stream);

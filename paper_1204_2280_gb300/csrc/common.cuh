@@ -55,15 +55,17 @@ constexpr int JUDGE_MAX = 4096;                        // sampled bodies of the 
 #define JUDGE_SPLIT_CFG 128
 #endif
 constexpr int JUDGE_SPLIT = JUDGE_SPLIT_CFG;            // source splits of the judge's direct sum
-#ifndef BUILD_THREADS_CFG
-#define BUILD_THREADS_CFG 1024
-#endif
-constexpr int BUILD_THREADS = BUILD_THREADS_CFG;       // threads per build block (multiple of 32, <= 1024)
-#ifndef BUILD_BPT_CFG
-#define BUILD_BPT_CFG 4
-#endif
-constexpr int BUILD_BPT = BUILD_BPT_CFG;               // bodies per thread of the build's analysis pass
-constexpr int BUILD_BODIES = BUILD_BPT * BUILD_THREADS;   // bodies per build block
+// Build blocks: of 1,024 bodies, one per thread, up to BUILD_SMALL_N bodies
+// (of 4,096 they would leave most SMs idle), else of 4,096, four per thread
+// (fewer halos, count rows and blocks).  Whole tree build, large / small
+// blocks (their counts added up by pass 3): 24 / 18 us at 2^12, 26 / 20 at
+// 2^15, 28 / 20 at 100,000, 30 / 22 at 2^18, 32 / 32 at 2^19, 40 / 50 at
+// 2^20 and 299 / 519 at 2^24.  Blocks of 512 gain no more and, with other
+// work on the GPU, cost steps of 100,000 bodies 0.5%.
+constexpr int BUILD_LARGE = 4096, BUILD_SMALL = 1024;
+constexpr long long BUILD_SMALL_N = 1 << 18;
+constexpr int build_bodies(long long n) { return n <= BUILD_SMALL_N ? BUILD_SMALL : BUILD_LARGE; }
+constexpr long long build_blocks(long long n) { return (n + build_bodies(n) - 1) / build_bodies(n); }
 constexpr int PACK_THREADS = 1024;                     // unpacked groups per group-packing block
 constexpr long long STAGE_MIN_FLOATS = 4096;           // staging area floor (getters stream cells through it)
 constexpr int ENTRY_ROW = NROWS;                       // build: entries per block (a row that is not scanned)
@@ -130,7 +132,7 @@ struct Ctx {
     // sizes
     long long n = 0, ncap = 0, ccap = 0;
     long long cells_hint = 0;         // cell count of the last tree the host read (0: none); sizes launches
-    int ntiles = 0, nbblocks = 0;     // sort tiles, build blocks
+    int ntiles = 0;                   // sort tiles
     bool hold_tile = false;           // testing aid on: the radix sort, whose tiles wait on one another
     int nsys = 1;                     // independent systems (contiguous body segments)
 
@@ -144,7 +146,7 @@ struct Ctx {
     uint32_t *vals = nullptr, *vals_alt = nullptr;   // vals ends as perm
     unsigned *tile_status = nullptr;                   // (SORT_PASSES + 1) * ntiles * SORT_RADIX
     // build
-    unsigned *blockcount = nullptr;  // BUILD_ROWS * nbblocks
+    unsigned *blockcount = nullptr;  // BUILD_ROWS x build blocks
     uint4 *build_entries = nullptr;  // per build block, the bodies that start cells (capacity n)
     uint2 *cell_body = nullptr, *cell_link = nullptr;
     uint8_t *cell_level = nullptr;

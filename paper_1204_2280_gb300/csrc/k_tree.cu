@@ -93,36 +93,39 @@ __device__ __forceinline__ int system_end(const DevState *__restrict__ st, const
 // levels.  Per block: cells per level (a difference array over lo..hi),
 // groups, and entries.
 constexpr int BH = 64;                              // halo: max(nleaf, ncrit)
-constexpr int BB = BUILD_BODIES;                    // bodies per block (BUILD_BPT per thread)
-constexpr int BTAB = BB + BH;                       // table positions [base - BH, base + BB)
-constexpr int BKEYS = BB + 2 * BH + 1;              // keys of [base - BH - 1, base + BB + BH)
 
+// BB bodies per block, BPT per thread.
+template <int BB, int BPT>
 struct MarkShared {
+    static constexpr int BTAB = BB + BH;            // table positions [base - BH, base + BB)
+    static constexpr int BKEYS = BB + 2 * BH + 1;   // keys of [base - BH - 1, base + BB + BH)
+    static constexpr int NT = BB / BPT;             // threads
     unsigned long long k[BKEYS];
     unsigned tab[2][BTAB];         // (D + 1) | (DG + 1) << 16, then maxima over 2^q positions
     unsigned e_t[BB];              // the block's entries: first body
     unsigned e_d[BB];              //   lo | hi << 8 | lg << 16 | kind << 24
     int cnt[MAX_LEVEL + 2];        // difference array of cells per level
-    unsigned wcnt[BUILD_BPT][BUILD_THREADS / 32];
+    unsigned wcnt[BPT][NT / 32];
     unsigned ngrp, ne;
     uint8_t sy[BKEYS];
 };
-
-size_t build_mark_smem_bytes() { return sizeof(MarkShared); }
 
 // End of the level-L run from body t (L >= 1), i.e. the first body after t
 // whose key differs from k[t] above level L: a binary search over the
 // block's keys and halo (the prefix shared with k[t] only shrinks along the
 // sorted keys; positions past n or in another system share nothing), then
 // the global search when the run reaches past the halo (identical keys at
-// the deepest level).
-__device__ __forceinline__ int run_end_local(const MarkShared &S, int k0, int base, int t, int L, int n,
-                                             const unsigned long long *__restrict__ sk, int send) {
+// the deepest level), which alone needs the end of t's system.
+template <int BB, int BPT>
+__device__ __forceinline__ int run_end_local(const MarkShared<BB, BPT> &S, int k0, int base, int t, int L, int n,
+                                             const unsigned long long *__restrict__ sk,
+                                             const DevState *__restrict__ st, const uint8_t *__restrict__ sysid,
+                                             bool multi) {
     const int last = base + BB + BH - 1;                     // last key in shared memory
     const unsigned long long kt = S.k[t - k0];
-    const uint8_t st = S.sy[t - k0];
-    auto inside = [&](int j) { return j < n && S.sy[j - k0] == st && key_cpl(kt, S.k[j - k0]) >= L; };
-    if (last > t && inside(last)) return run_end(sk, send, t, L);
+    const uint8_t sys = S.sy[t - k0];
+    auto inside = [&](int j) { return j < n && S.sy[j - k0] == sys && key_cpl(kt, S.k[j - k0]) >= L; };
+    if (last > t && inside(last)) return run_end(sk, multi ? system_end(st, sysid, t, n) : n, t, L);
     int lo = t, hi = last;                                    // inside(lo), !inside(hi)
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -140,16 +143,19 @@ __device__ __forceinline__ unsigned window_max(const unsigned *T, int it, int w,
     return m;
 }
 
-__global__ void __launch_bounds__(BUILD_THREADS)
+template <int BB, int BPT>
+__global__ void __launch_bounds__(BB / BPT)
 k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restrict__ sysid, int n, int nleaf,
              int ncrit, unsigned *blockcount, int nblocks, uint4 *entries, const DevState *__restrict__ st,
              bool multi) {
     extern __shared__ unsigned long long mark_smem[];
-    MarkShared &S = *reinterpret_cast<MarkShared *>(mark_smem);
-    if (st->status & ST_TIMEOUT) return;        // keys not sorted: skip the build
+    using Shared = MarkShared<BB, BPT>;
+    constexpr int NT = Shared::NT, BTAB = Shared::BTAB, BKEYS = Shared::BKEYS;
+    Shared &S = *reinterpret_cast<Shared *>(mark_smem);
+    const bool skip = st->status & ST_TIMEOUT;   // keys not sorted: skip the build
     const int base = blockIdx.x * BB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k0 = base - BH - 1;
-    for (int i = tid; i < BKEYS; i += BUILD_THREADS) {
+    for (int i = tid; i < BKEYS; i += NT) {
         const int j = k0 + i;
         const bool in = j >= 0 && j < n;
         S.k[i] = in ? sk[j] : 0ull;
@@ -157,13 +163,14 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
     }
     if (tid <= MAX_LEVEL + 1) S.cnt[tid] = 0;
     if (tid == 0) S.ngrp = 0u;
+    if (skip) return;
     __syncthreads();
     // with one system every body shares it: no system-id compare
     auto cpl = [&](int a, int b) {
         return multi ? body_cpl(S.k[a - k0], S.k[b - k0], S.sy[a - k0], S.sy[b - k0])
                      : key_cpl(S.k[a - k0], S.k[b - k0]);
     };
-    for (int i = tid; i < BTAB; i += BUILD_THREADS) {
+    for (int i = tid; i < BTAB; i += NT) {
         const int j = base - BH + i;             // table position
         int d = -1, dg = -1;
         if (j >= 0 && j < n) {
@@ -174,14 +181,14 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
     }
     __syncthreads();
 
-    // This thread's bodies t[h] = base + tid + h * BUILD_THREADS (h <
-    // BUILD_BPT): own l0, D, DG, then the window maxima from maxima over 2^qb
+    // This thread's bodies t[h] = base + tid + h * NT (h <
+    // BPT): own l0, D, DG, then the window maxima from maxima over 2^qb
     // positions, qb = floor(log2(min(nleaf, ncrit) + 1)) capped at 16 positions.
-    int t[BUILD_BPT], l0[BUILD_BPT];
-    unsigned own[BUILD_BPT];
+    int t[BPT], l0[BPT];
+    unsigned own[BPT];
 #pragma unroll
-    for (int h = 0; h < BUILD_BPT; h++) {
-        t[h] = base + tid + h * BUILD_THREADS;
+    for (int h = 0; h < BPT; h++) {
+        t[h] = base + tid + h * NT;
         own[h] = S.tab[0][t[h] - base + BH];
         l0[h] = (t[h] <= 0 || t[h] >= n) ? 0 : cpl(t[h] - 1, t[h]) + 1;
     }
@@ -191,14 +198,14 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
         const int hq = 1 << q;
         const unsigned *T = S.tab[cur];
         unsigned *U = S.tab[cur ^ 1];
-        for (int i = tid; i + 2 * hq <= BTAB; i += BUILD_THREADS) U[i] = __vmaxu2(T[i], T[i + hq]);
+        for (int i = tid; i + 2 * hq <= BTAB; i += NT) U[i] = __vmaxu2(T[i], T[i + hq]);
         __syncthreads();
         cur ^= 1;
     }
-    bool has[BUILD_BPT];
-    unsigned desc[BUILD_BPT];
+    bool has[BPT];
+    unsigned desc[BPT];
 #pragma unroll
-    for (int h = 0; h < BUILD_BPT; h++) {
+    for (int h = 0; h < BPT; h++) {
         const int it = t[h] - base + BH;
         const int winD = (int)(window_max(S.tab[cur], it, nleaf, qb) & 0xffffu);   // 1 + max D
         has[h] = t[h] < n && l0[h] <= MAX_LEVEL && (l0[h] == 0 || winD >= l0[h]);
@@ -217,18 +224,18 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
     }
     // compaction of the block's entries, in key order (slice h of the block's
     // bodies before slice h + 1)
-    unsigned m[BUILD_BPT];
+    unsigned m[BPT];
 #pragma unroll
-    for (int h = 0; h < BUILD_BPT; h++) {
+    for (int h = 0; h < BPT; h++) {
         m[h] = __ballot_sync(0xffffffffu, has[h]);
         if (lane == 0) S.wcnt[h][warp] = __popc(m[h]);
     }
     __syncthreads();
     if (warp == 0) {
-        constexpr int NW = BUILD_THREADS / 32;
+        constexpr int NW = NT / 32;
         unsigned carry = 0u;
 #pragma unroll
-        for (int h = 0; h < BUILD_BPT; h++) {
+        for (int h = 0; h < BPT; h++) {
             const unsigned v = lane < NW ? S.wcnt[h][lane] : 0u;
             unsigned x = v;
 #pragma unroll
@@ -243,7 +250,7 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
     }
     __syncthreads();
 #pragma unroll
-    for (int h = 0; h < BUILD_BPT; h++) {
+    for (int h = 0; h < BPT; h++) {
         if (has[h]) {
             const unsigned slot = S.wcnt[h][warp] + __popc(m[h] & ((1u << lane) - 1u));
             S.e_t[slot] = (unsigned)t[h];
@@ -252,7 +259,7 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
     }
     __syncthreads();
     const unsigned ne = S.ne;
-    for (unsigned e = (unsigned)tid; e < ne; e += BUILD_THREADS) {
+    for (unsigned e = (unsigned)tid; e < ne; e += NT) {
         // A leaf ends where the next entry starts (the first body after a
         // leaf starts a cell); a group at level lg < hi ends at the first
         // later entry that starts on a level <= lg.  Only at the end of the
@@ -260,8 +267,7 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
         const unsigned et = S.e_t[e], ed = S.e_d[e];
         const int elo = (int)(ed & 0xffu), ehi = (int)((ed >> 8) & 0xffu), elg = (int)((ed >> 16) & 0xffu);
         const int kind = (int)(ed >> 24);
-        const int send = system_end(st, sysid, (int)et, n);
-        const int lend = e + 1 < ne ? (int)S.e_t[e + 1] : run_end_local(S, k0, base, (int)et, ehi, n, sk, send);
+        const int lend = e + 1 < ne ? (int)S.e_t[e + 1] : run_end_local(S, k0, base, (int)et, ehi, n, sk, st, sysid, multi);
         const unsigned lcnt = (unsigned)lend - et;
         unsigned gcnt = 0u, ngrp = 0u;
         if (kind == 1) {
@@ -270,7 +276,7 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
             } else {
                 unsigned j = e + 1;
                 while (j < ne && (S.e_d[j] & 0xffu) > (unsigned)elg) j++;
-                const int gend = j < ne ? (int)S.e_t[j] : run_end_local(S, k0, base, (int)et, elg, n, sk, send);
+                const int gend = j < ne ? (int)S.e_t[j] : run_end_local(S, k0, base, (int)et, elg, n, sk, st, sysid, multi);
                 gcnt = (unsigned)gend - et;
             }
             ngrp = 1u;
@@ -299,7 +305,8 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
     }
 }
 
-// Pass 2: exclusive scan of each row over blocks (one block per row).
+// Pass 2: exclusive scan of each row over blocks (one block per row).  Not
+// launched for small blocks, whose counts pass 3 adds up itself.
 __global__ void __launch_bounds__(1024)
 k_build_scan(unsigned *blockcount, int nblocks, DevState *st) {
     __shared__ unsigned s_w[32];
@@ -344,10 +351,15 @@ k_build_scan(unsigned *blockcount, int nblocks, DevState *st) {
 // level r+1's first index: for an internal cell that is its first child, and
 // the children of a cell are the level-(r+1) cells between its cb and the
 // next cell's cb.  Leaves get their body count here.
-constexpr int WRITE_THREADS = 512;
+// FOLD (small blocks, so at most FOLD_MAX): the counts are not scanned yet; every block adds up the
+// rows' counts before it and in total (a few loads a lane and one launch
+// less: builds up to 2^18 bodies 2 us faster; at 2^20
+// 40 -> 37 us alone, but ensembles 0.2% slower).
+constexpr int FOLD_MAX = (int)(BUILD_SMALL_N / BUILD_SMALL), WRITE_THREADS = 512;   // (128 threads: 3 us slower at 2^12..2^17)
 
+template <bool FOLD>
 __global__ void __launch_bounds__(WRITE_THREADS)
-k_build_write(const uint4 *__restrict__ entries, int ncrit, const unsigned *__restrict__ blockcount, int nblocks,
+k_build_write(const uint4 *__restrict__ entries, int bb, int ncrit, const unsigned *__restrict__ blockcount, int nblocks,
               long long ccap, DevState *st, uint2 *cell_body, uint2 *cell_link, uint8_t *cell_level,
               uint32_t *cell_parent, uint32_t *cell_cb, uint2 *groups, uint8_t *group_lvl) {
     constexpr int NW = WRITE_THREADS / 32;
@@ -356,11 +368,34 @@ k_build_write(const uint4 *__restrict__ entries, int ncrit, const unsigned *__re
     __shared__ unsigned s_tot[NROWS];
     __shared__ int s_ok;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned ne = blockcount[(size_t)ENTRY_ROW * nblocks + blockIdx.x];
     if (st->status & ST_TIMEOUT) return;        // keys not sorted: skip the build
+    if (FOLD) {
+        for (int row = warp; row < NROWS; row += NW) {
+            const unsigned *cnt = blockcount + (size_t)row * nblocks;
+            unsigned before = 0u, all = 0u;
+#pragma unroll
+            for (int k = 0; k < FOLD_MAX / 32; k++) {
+                const int b = lane + 32 * k;
+                const unsigned v = b < nblocks ? cnt[b] : 0u;
+                all += v;
+                before += b < (int)blockIdx.x ? v : 0u;
+            }
+            all = __reduce_add_sync(0xffffffffu, all);
+            before = __reduce_add_sync(0xffffffffu, before);
+            if (lane == 0) {
+                s_tot[row] = all;
+                s_base[row] = before;
+                if (blockIdx.x == 0) st->row_total[row] = all;
+            }
+        }
+        __syncthreads();
+    }
     if (warp == 0) {                             // level offsets: one lane per row
         const bool lvl = lane <= MAX_LEVEL;
-        const unsigned tot = lane < NROWS ? st->row_total[lane] : 0u;
-        const unsigned bcnt = lane < NROWS ? blockcount[(size_t)lane * nblocks + blockIdx.x] : 0u;
+        const unsigned tot = lane >= NROWS ? 0u : FOLD ? s_tot[lane] : st->row_total[lane];
+        const unsigned bcnt = lane >= NROWS ? 0u
+                              : FOLD ? s_base[lane] : blockcount[(size_t)lane * nblocks + blockIdx.x];
         unsigned x = lvl ? tot : 0u;             // inclusive scan of the level totals
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -369,6 +404,7 @@ k_build_write(const uint4 *__restrict__ entries, int ncrit, const unsigned *__re
         }
         const unsigned run = __shfl_sync(0xffffffffu, x, MAX_LEVEL);   // all cells
         const unsigned excl = x - (lvl ? tot : 0u);
+        const unsigned ngr = __shfl_sync(0xffffffffu, tot, GROUP_ROW);
         if (lvl) s_base[lane] = excl + bcnt;
         if (lane == GROUP_ROW) s_base[GROUP_ROW] = bcnt;
         if (lvl && blockIdx.x == 0) st->level_start[lane] = excl;
@@ -380,19 +416,18 @@ k_build_write(const uint4 *__restrict__ entries, int ncrit, const unsigned *__re
                 // a guard): no cells and no groups, so that every later
                 // stage does nothing, and the error is reported
                 st->ncells = s_ok ? run : 0u;
-                st->ngroups = s_ok ? st->row_total[GROUP_ROW] : 0u;
+                st->ngroups = s_ok ? ngr : 0u;
                 if (!s_ok) atomicOr(&st->status, ST_CAPACITY);
             }
         }
     }
     __syncthreads();
     if (!s_ok) return;
-    const unsigned ne = blockcount[(size_t)ENTRY_ROW * nblocks + blockIdx.x];
     const unsigned lt = (1u << lane) - 1u;
     for (unsigned r0 = 0; r0 < ne; r0 += WRITE_THREADS) {   // rounds of entries (uniform)
         const unsigned i = r0 + (unsigned)tid;
         const bool valid = i < ne;
-        const uint4 e = valid ? entries[(size_t)blockIdx.x * BB + i] : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 e = valid ? entries[(size_t)blockIdx.x * bb + i] : make_uint4(0u, 0u, 0u, 0u);
         const int lo = valid ? (int)(e.w & 0xffu) : MAX_LEVEL + 1;
         const int hi = valid ? (int)((e.w >> 8) & 0xffu) : -1;
         const int lg = (int)((e.w >> 16) & 0xffu), kind = (int)(e.w >> 24);
@@ -477,8 +512,8 @@ __device__ __forceinline__ unsigned child_count(unsigned d, int l, const DevStat
 // and parent pointers of the children.
 __global__ void k_build_link(const DevState *__restrict__ st, const uint32_t *__restrict__ cell_cb,
                              const uint8_t *__restrict__ cell_level, uint2 *cell_link, uint32_t *cell_parent) {
-    if (st->status & ST_TIMEOUT) return;
-    const unsigned ncells = st->ncells;
+    const unsigned status = st->status, ncells = st->ncells;
+    if (status & ST_TIMEOUT) return;
     for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
         if (cell_link[c].y & LEAF_BIT) continue;
         const unsigned cb = cell_cb[c], nch = child_count(c, cell_level[c], st, cell_cb);
@@ -639,22 +674,32 @@ k_group_pack(DevState *st, const uint2 *__restrict__ graw, const uint8_t *__rest
     }
 }
 
+template <int BB, int BPT>
+static cudaError_t launch_mark(Ctx &c, int nb) {
+    static size_t attr_done[MAX_DEVICES] = {};
+    const size_t smem = sizeof(MarkShared<BB, BPT>);
+    const cudaError_t e = allow_dyn_smem((const void *)k_build_mark<BB, BPT>, smem, attr_done);
+    if (e != cudaSuccess) return e;
+    k_build_mark<BB, BPT><<<nb, BB / BPT, smem, c.stream>>>(
+        c.keys, c.sysid, (int)c.n, c.nleaf, c.ncrit, c.blockcount, nb, c.build_entries, c.st, c.nsys > 1);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_build(Ctx &c) {
     int n = (int)c.n;
-    static size_t attr_done[MAX_DEVICES] = {};
-    cudaError_t e = allow_dyn_smem((const void *)k_build_mark, sizeof(MarkShared), attr_done);
+    const int bb = build_bodies(n), nb = (int)build_blocks(n);
+    const bool pack = c.group_pack != 0, small = bb == BUILD_SMALL;
+    cudaError_t e = small ? launch_mark<BUILD_SMALL, 1>(c, nb) : launch_mark<BUILD_LARGE, 4>(c, nb);
     if (e != cudaSuccess) return e;
-    k_build_mark<<<c.nbblocks, BUILD_THREADS, sizeof(MarkShared), c.stream>>>(
-        c.keys, c.sysid, n, c.nleaf, c.ncrit, c.blockcount, c.nbblocks, c.build_entries, c.st, c.nsys > 1);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_build_scan<<<NROWS, 1024, 0, c.stream>>>(c.blockcount, c.nbblocks, c.st);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const bool pack = c.group_pack != 0;
-    k_build_write<<<c.nbblocks, WRITE_THREADS, 0, c.stream>>>(
-        c.build_entries, c.ncrit, c.blockcount, c.nbblocks, c.ccap, c.st, c.cell_body, c.cell_link, c.cell_level,
-        c.cell_parent, c.cell_cb, pack ? c.groups_raw : c.groups, pack ? c.group_lvl : nullptr);
+    if (!small) {
+        k_build_scan<<<NROWS, 1024, 0, c.stream>>>(c.blockcount, nb, c.st);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    const auto write = small ? k_build_write<true> : k_build_write<false>;
+    write<<<nb, WRITE_THREADS, 0, c.stream>>>(
+        c.build_entries, bb, c.ncrit, c.blockcount, nb, c.ccap, c.st, c.cell_body,
+        c.cell_link, c.cell_level, c.cell_parent, c.cell_cb, pack ? c.groups_raw : c.groups,
+        pack ? c.group_lvl : nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (pack) {

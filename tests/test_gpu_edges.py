@@ -307,3 +307,40 @@ def test_root_moments(sizes):
             bz.set_bodies(pos[off[k]:off[k + 1]], mass[off[k]:off[k + 1]]).build().multipoles()
             m1, q1 = B.bonsai_get_moments(bz.ctx)
         assert np.array_equal(mono[k], m1[0]) and np.array_equal(quad[k], q1[0])
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 4097, (1 << 18) - 1, (1 << 18) + 1])
+def test_build_blocks(n):
+    """Trees at the edges of the build's blocks (1,024 bodies up to 2^18, whose
+    counts pass 3 adds up, then 4,096), with runs of identical positions across block borders: cells, links,
+    levels and groups equal the oracle's, also for two systems and for few
+    bodies in a context that held many."""
+    import oracle
+    rng = np.random.default_rng(n)
+    pos = rng.normal(size=(n, 3)).astype(np.float32)
+    if n > 4000:
+        pos[rng.permutation(n)[:3000]] = pos[0]           # longer than a small block
+    few = rng.normal(size=(600, 3)).astype(np.float32)
+    half = n // 2
+
+    def alone(bz, p):
+        bz.set_bodies(p, np.ones(len(p), np.float32)).build()
+        key, _ = B.bonsai_get_keys(bz.ctx)
+        ref, t = oracle.build_tree(key, 8), B.bonsai_get_tree(bz.ctx)
+        for name in ("body_begin", "body_count", "child_begin", "nchild", "level"):
+            assert np.array_equal(t[name], getattr(ref, name)), name
+        groups, got = oracle.groups(ref, 16), B.bonsai_get_groups(bz.ctx)
+        assert np.array_equal(got[0], groups[0]) and np.array_equal(got[1], groups[1])
+        return ref.ncells, groups
+
+    with B.Bonsai(B.Config(nleaf=8, ncrit=16)) as bz:
+        alone(bz, pos)
+        alone(bz, few)
+        if n > 1:
+            (c0, g0), (c1, g1) = alone(bz, pos[:half]), alone(bz, pos[half:])
+            bz.set_bodies(pos, np.ones(n, np.float32)).set_systems([0, half, n]).build()
+            assert B.bonsai_get_sizes(bz.ctx)[1] == c0 + c1
+            got = B.bonsai_get_groups(bz.ctx)
+            assert np.array_equal(got[0], np.concatenate([g0[0], half + g1[0]]))
+            assert np.array_equal(got[1], np.concatenate([g0[1], g1[1]]))
+        bz.sync()
