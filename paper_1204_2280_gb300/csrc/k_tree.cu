@@ -13,7 +13,7 @@
 // launches: (1) per body, the levels on which it starts cells and its group,
 // compacted per block into a list of the bodies that start any (about one per
 // leaf), with counts per block and level; (2) scan of those counts over the
-// blocks; (3) per listed body, the index, first body, level and link of each
+// blocks (small trees: pass 3 adds them up); (3) per listed body, the index, first body, level and link of each
 // of its cells and its groups; (4) child counts and parents.  Internal
 // cells' body counts, which no stage of a step reads, are derived on demand
 // for the tree getter (k_internal_counts).
@@ -351,11 +351,12 @@ k_build_scan(unsigned *blockcount, int nblocks, DevState *st) {
 // level r+1's first index: for an internal cell that is its first child, and
 // the children of a cell are the level-(r+1) cells between its cb and the
 // next cell's cb.  Leaves get their body count here.
-// FOLD (small blocks, so at most FOLD_MAX): the counts are not scanned yet; every block adds up the
-// rows' counts before it and in total (a few loads a lane and one launch
-// less: builds up to 2^18 bodies 2 us faster; at 2^20
-// 40 -> 37 us alone, but ensembles 0.2% slower).
-constexpr int FOLD_MAX = (int)(BUILD_SMALL_N / BUILD_SMALL), WRITE_THREADS = 512;   // (128 threads: 3 us slower at 2^12..2^17)
+// FOLD (small blocks, so at most FOLD_MAX): the counts are not scanned yet;
+// every block adds up the rows' counts before it and in total (a few loads a
+// lane and one launch less: builds up to 2^18 bodies 2 us faster; at 2^20
+// 40 -> 37 us alone, steps the same).  Blocks of 128 threads for the few
+// entries of a small block: 3 us slower at 2^12..2^17.
+constexpr int FOLD_MAX = (int)(BUILD_SMALL_N / BUILD_SMALL), WRITE_THREADS = 512;
 
 template <bool FOLD>
 __global__ void __launch_bounds__(WRITE_THREADS)

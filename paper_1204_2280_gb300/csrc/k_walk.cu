@@ -24,7 +24,8 @@
 //    lane in 8 body slots and four phases, 24 body places where one body per
 //    lane would leave 8..15 of 32 lanes empty; groups of 33..64 bodies (larger
 //    ncrit) in one with two bodies per lane.  The bodies of a lane share
-//    every source read;
+//    every source read.  Small walks take such groups in two or three parts by
+//    as many warps instead, one launch in all (launch_walk);
 //  * each tile is summed in plain FP32 and added to the body's accumulators
 //    with Kahan compensation (one compensated add per tile and component).
 // Body-cell (monopole + traceless quadrupole, softened):
