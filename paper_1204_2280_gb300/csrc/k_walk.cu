@@ -756,9 +756,11 @@ struct SphWarp {
 // 8 / pi: the cubic spline's normalisation in three dimensions.
 constexpr float SPH_NORM = 2.546479089470325f;
 
-// n <= 64 sources from place head (0 or 64; n padded to a multiple of 8):
-// plain float32 sums per body in source order, then one compensated (Kahan)
-// add into the body's density.
+// n <= 64 sources from place head (0 or 64): plain float32 sums per body in
+// source order, then one compensated (Kahan) add into the body's density.
+// Places are tested eight at a time; the bits of those past n, which hold
+// sources of earlier tiles, are cleared (no position is far enough to be
+// nobody's neighbour: smoothing lengths have no upper limit).
 template <int NB>
 __device__ __forceinline__ void sph_tile(const SphWarp &R, int head, int n, const float4 (&me)[2],
                                          const float (&h2)[2], const float (&ih)[2], const bool (&live)[2],
@@ -789,7 +791,8 @@ __device__ __forceinline__ void sph_tile(const SphWarp &R, int head, int n, cons
                     in[half] = __funnelshift_l(__float_as_uint(d.y), in[half], 1);
                 }
             }
-            if (n_h < 32) in[half] = n_h > 0 ? in[half] << (32 - n_h) : 0u;
+            // the first source's bit highest; none past the last source
+            if (n_h < 32) in[half] = n_h > 0 ? (in[half] << (32 - ((n_h + 7) & ~7))) & ~(0xffffffffu >> n_h) : 0u;
         }
         if (!live[b]) in[0] = in[1] = 0u;
         cnt[b] += (unsigned)(__popc(in[0]) + __popc(in[1]));
@@ -949,12 +952,7 @@ k_sph_walk(const DevState *__restrict__ stc, DevState *st, const uint2 *__restri
             }
             __syncwarp();
         }
-        if (nsrc > 0) {
-            const int pad = -nsrc & 7;                  // sources far away, no body's neighbours
-            if (lane < pad) put_body_at<SPH_RP>(R.src[0], head + nsrc + lane, make_float4(1e18f, 1e18f, 1e18f, 0.f));
-            __syncwarp();
-            sph_eval(ng > 32, R, head, nsrc + pad, me, h2, ih, live, rho, comp, cnt);
-        }
+        if (nsrc > 0) sph_eval(ng > 32, R, head, nsrc, me, h2, ih, live, rho, comp, cnt);
 #pragma unroll
         for (int b = 0; b < 2; b++) {
             if (live[b]) {

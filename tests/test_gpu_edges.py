@@ -114,6 +114,25 @@ def test_sph_candidate_rings(n, ncrit):
         assert np.array_equal(cnt, ref[1]) and np.abs(rho / ref[0] - 1.0).max() <= 2e-5
 
 
+@pytest.mark.parametrize("n", [1, 33, 700])
+@pytest.mark.parametrize("scale,h", [(1.0, 1e19), (1.0, np.inf), (1e17, 2e17)])
+def test_sph_counts_bodies_only(n, scale, h):
+    """Neighbour counts where no finite place is out of reach (h^2 near and
+    past the largest float: every body is a neighbour) and for bodies about
+    1e18 from the origin: the oracle's, whatever the last ring of candidates
+    holds past its end."""
+    import oracle
+    rng = np.random.default_rng(n)
+    pos = (rng.normal(size=(n, 3)) * scale + (1e18 if scale > 1.0 else 0.0)).astype(np.float32)
+    mass, hs = np.ones(n, np.float32), np.full(n, h, np.float32)
+    rho, cnt = np.zeros(n, np.float32), np.zeros(n, np.int32)
+    with B.Bonsai(B.Config(ncrit=32)) as bz:
+        bz.set_bodies(pos, mass).build()
+        B.bonsai_sph_density(bz.ctx, hs, rho, cnt)
+        bz.sync()
+    assert np.array_equal(cnt, oracle.sph_density(pos, mass, hs)[1])
+
+
 @pytest.mark.parametrize("n", [(1 << 18) - 1, 1 << 18, (1 << 18) + 1, 300001])
 def test_caller_order_outputs(n):
     """Positions, velocities, forces and potentials in caller order on both
