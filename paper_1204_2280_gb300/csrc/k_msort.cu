@@ -12,9 +12,9 @@
 //     rounds of merges in shared memory, each thread finding its share by
 //     merge path;
 //   * merge: a block writes one tile of the merged run; two warps find the
-//     tile's ends in the two runs with 32-way searches (three or four rounds
-//     of dependent loads), the tile's keys go to shared memory and each
-//     thread merges MS_IPT of them;
+//     tile's ends in the two runs with 32-way searches (three rounds of
+//     dependent loads for runs of 4,608 keys, five for 2^21), the tile's keys
+//     go to shared memory and each thread merges MS_IPT of them;
 //   * the launch that finishes the order also moves the bodies (positions,
 //     velocities, ids) instead of writing the permutation for a further pass.
 // No block waits on another.  MS_IPT is odd, so that the threads' runs of
@@ -42,15 +42,14 @@ __device__ __forceinline__ int merge_path(const u64 *a, int na, const u64 *b, in
 }
 
 // The same over global memory by a whole warp: 32 places at a time.
-__device__ __forceinline__ int merge_path_warp(const u64 *__restrict__ a, int na, const u64 *__restrict__ b, int nb,
-                                               int d, int lane) {
+__device__ __forceinline__ int merge_path_warp(const u64 *a, int na, const u64 *b, int nb, int d, int lane) {
     int lo = max(0, d - nb), hi = min(d, na);
     while (lo < hi) {
         const int len = hi - lo;
         const bool few = len <= 32;
         const int at = few ? lane : (int)((long long)(lane + 1) * len / 33);
         const int mid = lo + at;
-        const bool before = (!few || lane < len) && __ldg(a + mid) <= __ldg(b + d - 1 - mid);
+        const bool before = (!few || lane < len) && a[mid] <= b[d - 1 - mid];
         const int c = __popc(__ballot_sync(0xffffffffu, before));
         if (few) return lo + c;
         const int m_lo = (int)((long long)c * len / 33), m_hi = (int)((long long)(c + 1) * len / 33);
@@ -82,9 +81,8 @@ __device__ __forceinline__ void serial_merge(const u64 *s, int a, int aend, int 
 }
 
 struct ReorderArgs {
-    const float4 *__restrict__ pin;
-    const float4 *__restrict__ vin;
-    const uint32_t *__restrict__ idin;
+    const float4 *pin, *vin;
+    const uint32_t *idin;
     float4 *pout, *vout;
     uint32_t *idout;
 };
@@ -101,9 +99,13 @@ __device__ __forceinline__ void move_body(const ReorderArgs &r, int to, uint32_t
 // launch): a kernel lets its successor be set up while it runs, and waits
 // until its predecessor is complete and its writes are visible (a hardware
 // wait, no polling) before it reads.  As every kernel of the chain waits for
-// the one before, all earlier work is complete too.  A static sort of 65,536
-// keys 71 -> 65 us; the same for the build's and the multipoles' launches
-// measured no gain at 2^12..2^17 and 0.5% more time at 2^20.
+// the one before, all earlier work is complete too.  The buffers that the
+// chain writes change while its later kernels are already resident, so these
+// kernels read memory by ordinary loads only, which the wait orders and the
+// compiler keeps behind it: no const __restrict__ pointers and no __ldg, whose
+// data must not change while a kernel lives.  A static sort of 65,536 keys
+// 71 -> 65 us; the same for the build's and the multipoles' launches measured
+// no gain at 2^12..2^17 and 0.5% more time at 2^20.
 __device__ __forceinline__ void follow_previous() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -222,8 +224,7 @@ constexpr size_t MS_MERGE_SMEM = (size_t)(MS_TILE + MS_SLACK) * (sizeof(u64) + s
 // runs twice as long; block t writes outputs [t MS_TILE, (t + 1) MS_TILE).
 template <bool MOVE>
 __global__ void __launch_bounds__(MS_THREADS, 2)
-k_merge(const u64 *__restrict__ kin, const uint32_t *__restrict__ vin, u64 *kout, uint32_t *vout, int n, int run,
-        ReorderArgs r) {
+k_merge(const u64 *kin, const uint32_t *vin, u64 *kout, uint32_t *vout, int n, int run, ReorderArgs r) {
     extern __shared__ u64 ms_smem[];
     u64 *s_k = ms_smem;
     uint32_t *s_v = reinterpret_cast<uint32_t *>(ms_smem + MS_TILE + MS_SLACK);
