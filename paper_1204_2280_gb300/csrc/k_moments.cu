@@ -475,8 +475,10 @@ k_mom_combine(MomArrays a) {
                 c = p; plk = pl; lv = plv; p = gp;
             }
         }
-        // the lane's acquire and the warp barrier of the ballot make the
-        // children's moments visible to the whole warp
+        // A lane that completed a root has acquired its children's moments;
+        // the barrier passes that on to the other lanes (votes and shuffles
+        // order no memory).
+        __syncwarp();
         for (unsigned rm = __ballot_sync(0xffffffffu, root); rm; rm &= rm - 1u) {
             const int src = __ffs(rm) - 1;
             root_cell<REFIT>(__shfl_sync(0xffffffffu, c, src),

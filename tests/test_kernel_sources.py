@@ -26,3 +26,13 @@ def test_no_read_only_loads_in_overlapping_launches():
         for word in ("__restrict__", "__ldg", "__ldcg", "__ldcs", "__ldca", "ld.global.nc"):
             assert word not in code, (path.name, word)
     assert found == ["k_msort.cu"]
+
+
+def test_barrier_between_arrival_and_root():
+    """A root's children are acquired by one lane and read by its whole warp:
+    a warp barrier, which alone orders memory between lanes, stands between
+    the arrival on the parent and the work on the roots."""
+    code = _code(CSRC / "k_moments.cu")
+    arrival = code.index("atom_add_acq_rel_gpu(&a.cell_done")
+    between = code[arrival:code.index("root_cell<REFIT>(", arrival)]
+    assert "__syncwarp();" in between
