@@ -19,6 +19,18 @@ static thread_local std::string g_create_err;
 namespace bonsai {
 // Errors of calls without a context (bonsai_create, bonsai_sort_keys_static).
 void set_global_error(const char *msg) { g_create_err = msg; }
+
+// Whether a caller has ever captured this context's launches (every call
+// that launches asks, so that no capture goes unseen).  Calls made later
+// cannot know when such a graph is replayed, and it uses the walk's queues and
+// the domain box: from then on no call leaves out what an earlier one has
+// done, and none does a later one's part in advance.
+bool seen_capture(Ctx &c) {
+    if (c.captured) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c.stream, &cs) != cudaSuccess) { cudaGetLastError(); return true; }
+    return c.captured = cs != cudaStreamCaptureStatusNone;
+}
 }  // namespace bonsai
 
 static int fail(bonsai_ctx *ctx, int code, const std::string &what, cudaError_t e = cudaSuccess) {
@@ -154,15 +166,6 @@ cudaError_t run_cached(Ctx &c, CallGraph &g, const long long *key, int nkey, F b
     for (int i = 0; i < nkey; i++) g.key[i] = key[i];
     g.nkey = nkey;
     return body();
-}
-
-// Whether the caller is capturing the stream: what a call may skip because an
-// earlier call has done it must then be in the captured launches all the
-// same, since they are replayed without that call.
-bool caller_captures(Ctx &c) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c.stream, &cs) != cudaSuccess) { cudaGetLastError(); return true; }
-    return cs != cudaStreamCaptureStatusNone;
 }
 
 long long fbits(float x) {
@@ -373,7 +376,7 @@ int bonsai_build(bonsai_ctx *ctx) {
     if (!ctx) return BONSAI_ERR_INVALID_ARG;
     Ctx &c = ctx->c;
     if (!c.have_bodies) return fail(ctx, BONSAI_ERR_NOT_READY, "bonsai_build: no bodies");
-    const bool again = c.built, boxed = c.dom_ready && !caller_captures(c);
+    const bool again = c.built, boxed = !seen_capture(c) && c.dom_ready;
     const long long key[] = {c.n, c.arena_gen, c.nsys, c.nleaf, c.ncrit, c.group_pack, c.max_spin, again,
                              c.hold_tile, boxed};
     CK(run_cached(c, c.build_graph, key, (int)(sizeof key / sizeof key[0]), [&]() -> cudaError_t {
@@ -408,7 +411,8 @@ int bonsai_multipoles(bonsai_ctx *ctx) {
     // bodies changes little); only a context without one reads it back.
     if (c.cells_hint == 0) CK(refresh_cells_hint(c));
     // the totals of a walk stay readable until the next one
-    const bool reset = !c.have_acc;
+    const bool reset = !seen_capture(c) && !c.have_acc;
+    c.walk_ready = false;
     const long long key[] = {c.n, c.arena_gen, c.nsys, c.cells_hint, reset};
     CK(run_cached(c, c.mom_graph, key, (int)(sizeof key / sizeof key[0]), [&]() { return launch_multipoles(c, reset); }));
     c.walk_ready = reset;
@@ -440,14 +444,14 @@ int bonsai_forces(bonsai_ctx *ctx, float theta, float eps, float *acc, float *po
         return fail(ctx, BONSAI_ERR_NOT_READY, "bonsai_forces: call bonsai_build and bonsai_multipoles first");
     c.theta = theta;
     c.eps = eps;
-    const bool ready = c.walk_ready && !caller_captures(c);   // right after the multipoles
+    const bool ready = !seen_capture(c) && c.walk_ready;      // right after the multipoles
+    c.walk_ready = false;
     const long long key[] = {c.n, c.arena_gen, c.nsys, c.ncrit, c.group_pack, c.walk_warps, c.list_capacity,
                              c.max_spin, fbits(theta), fbits(eps), c.block_kmax, ready};
     CK(run_cached(c, c.forces_graph, key, (int)(sizeof key / sizeof key[0]), [&]() -> cudaError_t {
         const cudaError_t e = ready ? cudaSuccess : launch_reset(c, RESET_WALK);
         return e != cudaSuccess ? e : pipeline_forces(c, theta, eps);
     }));
-    c.walk_ready = false;
     c.have_acc = true;
     if (acc || pot) {
         if (on_device) {
@@ -474,6 +478,7 @@ int bonsai_step(bonsai_ctx *ctx, float dt) {
         if (!c.moments_ready && (r = bonsai_multipoles(ctx))) return r;
         if ((r = bonsai_forces(ctx, c.theta, c.eps, nullptr, nullptr, 1))) return r;
     }
+    seen_capture(c);
     // The first step with a given (dt, theta, eps, N) runs eagerly; the second
     // captures the step into a CUDA graph, later ones replay it.
     const bool same = c.graph_dt == dt && c.graph_theta == c.theta && c.graph_eps == c.eps &&

@@ -439,6 +439,7 @@ int bonsai_forces_learned(bonsai_ctx *ctx, float eps, float *acc, float *pot, in
     if (!c.moments_ready)
         return cfail(ctx, BONSAI_ERR_NOT_READY, "bonsai_forces_learned: call bonsai_build and bonsai_multipoles first");
     if (!(eps > 0.f)) return cfail(ctx, BONSAI_ERR_INVALID_ARG, "bonsai_forces_learned: eps > 0");
+    seen_capture(c);
     c.walk_ready = false;
     CCK(launch_reset(c));
     CCK(pipeline_learned_forces(c, eps));

@@ -49,6 +49,7 @@ int bonsai_sph_density(bonsai_ctx *ctx, const float *h, float *rho, int32_t *nng
     if (!c.built || !c.tree_fresh)
         return sfail(ctx, BONSAI_ERR_NOT_READY, "bonsai_sph_density: needs a tree built from the current positions "
                                                 "(bonsai_build or bonsai_step)");
+    seen_capture(c);
     c.walk_ready = false;            // this pass uses the walk's queue
     const int n = (int)c.n;
     // scratch in the learned path's feature array (12 floats per body):

@@ -175,6 +175,7 @@ struct Ctx {
     // pipeline state
     bool dom_ready = false;          // the domain box of the loaded bodies is on the device (one system, no build yet)
     bool walk_ready = false;         // the walk queues are reset since the last walk
+    bool captured = false;           // a caller has captured launches of this context (seen_capture)
     bool have_bodies = false, built = false, moments_ready = false, have_acc = false;
     long long arena_limit = 0;       // bytes; 0: no cap on the body arena
     bool tree_fresh = false;         // the tree was built from the current positions (no refit since)
@@ -276,6 +277,7 @@ __device__ __forceinline__ unsigned long long key_prefix(unsigned long long k, i
 }
 
 // ---- launchers (host) ------------------------------------------------------
+bool seen_capture(Ctx &c);
 cudaError_t launch_reset(Ctx &c, int what = RESET_DOMAIN | RESET_SORT | RESET_WALK);
 cudaError_t launch_domains(Ctx &c);
 cudaError_t launch_fill_sysid(Ctx &c);

@@ -246,6 +246,59 @@ def test_domain_of_loaded_bodies(n):
         bz.sync()
 
 
+@pytest.mark.parametrize("call,when", [("forces", "before forces"), ("sph", "before forces"), ("all", "before forces"),
+                                       ("learned", "before build"), ("learned", "before forces"),
+                                       ("multipoles", "after forces")])
+def test_replays_between_calls(call, when):
+    """A graph of the context's calls that its caller captured, replayed
+    between direct calls: it uses the walk's queues and the domain box, and the
+    direct calls that follow (another opening angle) give what they give
+    without it, with their own interaction totals."""
+    import torch
+    n = 20000
+    rng = np.random.default_rng(8)
+    pos = torch.from_numpy(rng.normal(size=(n, 3)).astype(np.float32)).cuda()
+    mass, h = torch.full((n,), 1.0 / n, device="cuda"), torch.full((n,), 0.2, device="cuda")
+    ref, acc, out = (torch.zeros(n, 3, device="cuda") for _ in range(3))
+    rho, cnt = torch.zeros(n, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    with B.Bonsai(B.Config(ncrit=32)) as bz:
+        bz.set_bodies(pos, mass).build().multipoles().forces(0.5, 0.01, ref)
+        tot = B.bonsai_get_counts(bz.ctx)[2]
+        bz.sync()
+    s, net = torch.cuda.Stream(), B.MLP(0)
+    with B.Bonsai(B.Config(ncrit=32), s.cuda_stream) as bz:
+        B.bonsai_set_learned(bz.ctx, net, 1.0, 0.9, 1e30)
+        run = dict(forces=lambda: bz.forces(0.9, 0.01, acc), multipoles=bz.multipoles,
+                   sph=lambda: B.bonsai_sph_density(bz.ctx, h, rho, cnt),
+                   learned=lambda: B.bonsai_forces_learned(bz.ctx, 0.01, acc),
+                   all=lambda: bz.build().multipoles().forces(0.9, 0.01, acc))[call]
+        for _ in range(2):
+            bz.set_bodies(pos, mass).build().multipoles()
+            run()                                        # direct: sets up what a capture may not
+        bz.set_bodies(pos, mass).build().multipoles().sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s, capture_error_mode="thread_local"):
+            run()
+
+        def replay(now):
+            if now == when:
+                with torch.cuda.stream(s):
+                    g.replay()
+
+        for _ in range(3):                               # direct launches, captured and replayed ones
+            out.zero_()
+            torch.cuda.synchronize()
+            bz.set_bodies(pos, mass)
+            replay("before build")
+            bz.build().multipoles()
+            replay("before forces")
+            bz.forces(0.5, 0.01, out)
+            replay("after forces")
+            assert B.bonsai_get_counts(bz.ctx)[2] == tot
+            bz.sync()
+            assert torch.equal(out, ref)
+
+
 @pytest.mark.parametrize("ncrit,pack,n", [(64, 0, 1), (64, 0, 33), (64, 0, 65), (33, 0, 500), (64, 1, 3000),
                                           (64, 0, 12000), (48, 1, 20000), (64, 1, (1 << 18) - 3), (32, 1, 17),
                                           (32, 0, 500), (32, 1, 24), (32, 1, 9000), (24, 1, 30000), (32, 1, 65536)])
