@@ -22,9 +22,9 @@ void set_global_error(const char *msg) { g_create_err = msg; }
 
 // Whether a caller has ever captured this context's launches (every call
 // that launches asks, so that no capture goes unseen).  Calls made later
-// cannot know when such a graph is replayed, and it uses the walk's queues and
-// the domain box: from then on no call leaves out what an earlier one has
-// done, and none does a later one's part in advance.
+// cannot know when such a graph is replayed, and it uses the walk's queues,
+// the domain box and the judge's sample: from then on no call leaves out what
+// an earlier one has done, and none does a later one's part in advance.
 bool seen_capture(Ctx &c) {
     if (c.captured) return true;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

@@ -35,12 +35,15 @@ __global__ void k_judge_targets(uint32_t *targets, int ntar, long long n) {
     if (k < ntar) targets[k] = (uint32_t)(((long long)k * n) / ntar);
 }
 
-// Stratified judge sample: every (n / ntar)-th body in key order.
+// Stratified judge sample: every (n / ntar)-th body in key order.  It is kept
+// while the number of bodies stays, unless a caller's graph may have filled it
+// or left it out.
 cudaError_t launch_judge_targets(Ctx &c) {
     const int ntar = (int)(c.n < JUDGE_MAX ? c.n : JUDGE_MAX);
-    if (c.judge_n == ntar) return cudaSuccess;
-    k_judge_targets<<<(ntar + 255) / 256, 256, 0, c.stream>>>(c.judge_targets, ntar, c.n);
+    if (!c.captured && c.judge_n == ntar && c.judge_bodies == c.n) return cudaSuccess;
     c.judge_n = ntar;
+    c.judge_bodies = c.n;
+    k_judge_targets<<<(ntar + 255) / 256, 256, 0, c.stream>>>(c.judge_targets, ntar, c.n);
     return cudaGetLastError();
 }
 

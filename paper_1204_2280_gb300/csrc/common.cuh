@@ -206,7 +206,8 @@ struct Ctx {
     uint32_t *judge_targets = nullptr;   // JUDGE_MAX sorted positions
     float4 *judge_partial = nullptr;     // JUDGE_SPLIT x JUDGE_MAX
     float4 *judge_direct = nullptr;      // JUDGE_MAX
-    int judge_n = 0;                     // targets in use
+    int judge_n = 0;                     // targets in use (0: none filled)
+    long long judge_bodies = 0;          // bodies they are a sample of
 
     std::string err;
 };

@@ -209,6 +209,27 @@ def test_judge_sizes(n):
     assert abs(p - ref) <= 1e-4 * ref + 1e-6
 
 
+@pytest.mark.parametrize("sizes", [(30001, 5000, 20000, 3000, 4500), (9000, 4096, 9000, 4095)])
+def test_judge_other_bodies(sizes):
+    """One context judged with one set of bodies and then with smaller and
+    larger ones: each judgement samples the bodies of its own set (p99 against
+    the oracle's direct sum at them, as above)."""
+    import oracle
+    with B.Bonsai(B.Config(ncrit=64)) as bz:
+        for n in sizes:
+            rng = np.random.default_rng(n)
+            pos, mass = rng.normal(size=(n, 3)).astype(np.float32), np.full(n, 1.0 / n, np.float32)
+            acc = np.zeros((n, 3), np.float32)
+            bz.set_bodies(pos, mass).build().multipoles().forces(1.1, 0.05, acc)
+            p = B.bonsai_judge(bz.ctx, 0.05)
+            t = min(n, 4096)
+            ids = B.bonsai_get_keys(bz.ctx)[1][(np.arange(t, dtype=np.int64) * n) // t].astype(np.int64)
+            a, _ = oracle.direct(pos, mass, 0.05, ids)
+            ref = np.percentile(np.linalg.norm(acc[ids] - a, axis=1) / np.linalg.norm(a, axis=1), 99)
+            assert abs(p - ref) <= 1e-4 * ref + 1e-6
+        bz.sync()
+
+
 @pytest.mark.parametrize("n", [1, 255, 257, 5000, 1216 * 256 + 1])
 def test_domain_of_loaded_bodies(n):
     """The domain box that loading leaves for the first build (block boxes,
