@@ -161,8 +161,10 @@ cudaError_t launch_direct(Ctx &c, const uint32_t *targets, int ntar, float eps, 
 // default), and the fallback flag p99 > budget.  One block of 1024 threads;
 // the two order statistics by bisection on the errors' bits (non-negative
 // floats order as their bits), one block count per bit: 38 us with a bitonic
-// sort of the 4096 errors, 18 us here.  Skipped by the gate, it leaves the
-// last judgement (p99 and flag) in place.
+// sort of the 4096 errors, 18 us here.  An error that is not finite (forces
+// that a diverged network made NaN) ranks as infinite, above every other and
+// below the places of absent targets, so that p99 is over every finite budget.
+// Skipped by the gate, it leaves the last judgement (p99 and flag) in place.
 __global__ void __launch_bounds__(1024)
 k_judge_p99(const float4 *__restrict__ acc4, const uint32_t *__restrict__ targets, int ntar,
             const float4 *__restrict__ direct, float budget, DevState *st, const unsigned *__restrict__ gate) {
@@ -173,14 +175,15 @@ k_judge_p99(const float4 *__restrict__ acc4, const uint32_t *__restrict__ target
 #pragma unroll
     for (int k = 0; k < PER; k++) {
         const int i = threadIdx.x + k * 1024;
-        float e = INFINITY;
+        v[k] = 0x7fffffffu;
         if (i < ntar) {
             const float4 a = acc4[targets[i]], d = direct[i];
             const float ex = a.x - d.x, ey = a.y - d.y, ez = a.z - d.z;
+            const float en = sqrtf(ex * ex + ey * ey + ez * ez);
             const float dn = sqrtf(d.x * d.x + d.y * d.y + d.z * d.z);
-            e = dn > 0.f ? sqrtf(ex * ex + ey * ey + ez * ez) / dn : 0.f;
+            const float e = dn == 0.f && en < INFINITY ? 0.f : en / dn;
+            v[k] = __float_as_uint(e < INFINITY ? e : INFINITY);
         }
-        v[k] = __float_as_uint(e) & 0x7fffffffu;
     }
     if (threadIdx.x == 0) s_next = 0xffffffffu;
     auto at_most = [&](unsigned x) {              // errors <= x, block-wide
@@ -204,9 +207,10 @@ k_judge_p99(const float4 *__restrict__ acc4, const uint32_t *__restrict__ target
     __syncthreads();
     if (threadIdx.x == 0) {
         const float v0 = __uint_as_float(lo), v1 = tie ? v0 : __uint_as_float(s_next);
-        const float p99 = v0 + (pos - (float)i0) * (v1 - v0);
+        const float f = pos - (float)i0;
+        const float p99 = v1 < INFINITY ? v0 + f * (v1 - v0) : f > 0.f ? v1 : v0;
         st->judge_p99 = p99;
-        st->fallback = p99 > budget ? 1u : 0u;
+        st->fallback = p99 <= budget ? 0u : 1u;
     }
 }
 

@@ -230,6 +230,26 @@ def test_judge_other_bodies(sizes):
         bz.sync()
 
 
+@pytest.mark.parametrize("n", [1, 300, 5000])
+def test_nan_correction_falls_back(n):
+    """A network whose outputs are NaN is rejected by the judge at every finite
+    budget: the forces are the fine walk's, bit for bit."""
+    rng = np.random.default_rng(n)
+    pos, mass = rng.normal(size=(n, 3)).astype(np.float32), np.full(n, 1.0 / n, np.float32)
+    net = B.MLP(0)
+    P, norm = net.get_params()
+    P[-B.MLP_OUT:] = np.nan                              # the output layer's biases
+    net.set_params(P, norm)
+    fine, a = np.zeros((n, 3), np.float32), np.zeros((n, 3), np.float32)
+    with B.Bonsai(B.Config(ncrit=64)) as bz:
+        bz.set_bodies(pos, mass).build().multipoles().forces(0.5, 0.01, fine)
+        for budget in (1.0, 1e30):
+            B.bonsai_set_learned(bz.ctx, net, 1.0, 0.5, budget)
+            B.bonsai_forces_learned(bz.ctx, 0.01, a)
+            assert B.bonsai_get_judge(bz.ctx) == (np.inf, True) and np.array_equal(a, fine)
+        bz.sync()
+
+
 @pytest.mark.parametrize("n", [1, 255, 257, 5000, 1216 * 256 + 1])
 def test_domain_of_loaded_bodies(n):
     """The domain box that loading leaves for the first build (block boxes,
