@@ -98,7 +98,8 @@ def kernels_per_step(ncrit, group_pack=0, n=None):
     (+2 for sibling packing of the groups), multipoles in two passes (leaves,
     then internal cells), walk (a second
     instantiation when groups may exceed 16 bodies: three bodies per lane for
-    17..24, two for more than 32; up to 2^16 and 2^18 bodies one launch), kick.
+    17..24, two for more than 32; up to 2^16 and 2^18 bodies one launch, but two
+    for packed groups of more than 32 below 20,000 bodies), kick.
     The build has one less up to 2^18 bodies.  (The start-list reset before the
     multipoles is a memset node, not a kernel.)"""
     order = 11                                # domains, keys, 8 radix passes, reorder
@@ -106,7 +107,8 @@ def kernels_per_step(ncrit, group_pack=0, n=None):
         order = 1 + merge_launches(n)
     second = ncrit > 16                       # a second walk launch
     if n is not None:
-        second = second and n > (1 << 18 if ncrit > 32 else 1 << 16)    # else parts in one launch
+        # else parts in one launch
+        second = second and (n > (1 << 18 if ncrit > 32 else 1 << 16) or ncrit > 32 and group_pack and n < 20000)
     scan = n is None or n > 1 << 18           # else pass 3 of the build adds the counts up itself
     return 9 + scan + order + second + (2 if group_pack else 0)
 

@@ -662,20 +662,33 @@ static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned 
     return cudaGetLastError();
 }
 
-// Up to these many bodies the groups of a second instantiation are walked in
-// parts by the first.  Each part traverses the tree, but a group's chain of
-// tiles is shorter, the kernel has 24 warps per SM instead of 12 or 16 and no
-// second launch follows: with few groups per warp the longest chain decides.
-// Evaluations, two launches / parts: groups of 33..64 (ncrit 64) 74 / 68 us at
-// 2^12, 112 / 92 at 2^14, 209 / 191 at 2^16, 592 / 591 at 2^18, 2251 / 2280 at
-// 2^20 (theta 0.5, 200,003 bodies: 1253 / 1142); groups of 17..24 (ncrit 32,
-// packed) 79 / 72 at 2^12, 125 / 120 at 2^15, 194 / 191 at 2^16, 300 / 320 at
-// 2^17.  Beyond, the repeated traversals cost more.
+// Between these numbers of bodies the groups of a second instantiation are
+// walked in parts by the first.  Each part traverses the tree, but the kernel
+// has 24 warps per SM instead of 12 or 16 and no second launch follows.  Forces,
+// two launches / parts, us (Plummer spheres, theta 0.75; 0.5 and 1 and the
+// walk with features change by the same factors):
+//   groups of 33..64: ncrit 64 unpacked 82 / 84 at 2^12, 108 / 99 at 2^13,
+//   180 / 167 at 2^15, 231 / 192 at 2^16, 335 / 291 at 2^17, 556 / 538 at 2^18,
+//   beyond which the repeated traversals cost more (evaluations at 2^20: 2251 /
+//   2280); ncrit 64 packed, where nearly every group is so large, 144 / 169 at
+//   2^12, 123 / 131 at 2^14, 161 / 155 at 24,000, 167 / 160 at 2^15, 334 / 311 at
+//   2^17, 574 / 546 at 2^18: below 20,000 bodies one group's chain decides, and
+//   two bodies per lane hide its latency better than two warps of one;
+//   groups of 17..24: ncrit 32 unpacked 71 / 65 at 2^12, 108 / 104 at 2^14,
+//   142 / 124 at 2^15, 204 / 190 at 2^16; packed 82 / 74 at 2^12, 114 / 126 at
+//   2^14, 130 / 150 at 24,000, 141 / 152 at 2^15, 166 / 163 at 50,000, 192 / 178
+//   at 2^16, 300 / 320 at 2^17.  Packed sizes in between lose for a walk alone,
+//   where all parts run at once and slow one another down, but win when other
+//   contexts share the GPU (evaluations in turn in three contexts: 86 / 82 at
+//   2^14, 98 / 94 at 24,000, 123 / 108 at 2^15, 147 / 124 at 40,000).
 #ifndef WALK_SPLIT3_MAX_N
 #define WALK_SPLIT3_MAX_N (1 << 16)
 #endif
 #ifndef WALK_SPLIT_MAX_N
 #define WALK_SPLIT_MAX_N (1 << 18)
+#endif
+#ifndef WALK_SPLIT_PACKED_MIN_N
+#define WALK_SPLIT_PACKED_MIN_N 20000
 #endif
 
 // One persistent launch per instantiation that can receive groups (group
@@ -704,7 +717,8 @@ cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features, const uns
                         : launch_walk_t<1, false, false>(c, theta, eps, gate, three, st);
     };
     const int second = c.ncrit >= WALK_BPL2_FROM ? 2 : three ? 3 : 0;
-    if (second == 2 && c.block_kmax < 0 && c.n <= WALK_SPLIT_MAX_N)
+    if (second == 2 && c.block_kmax < 0 && c.n <= WALK_SPLIT_MAX_N &&
+        (c.group_pack == 0 || c.n >= WALK_SPLIT_PACKED_MIN_N))
         return features ? launch_walk_t<1, true, false, 2>(c, theta, eps, gate, false, c.stream)
                         : launch_walk_t<1, false, false, 2>(c, theta, eps, gate, false, c.stream);
     if (second == 3 && c.block_kmax < 0 && c.n <= WALK_SPLIT3_MAX_N)

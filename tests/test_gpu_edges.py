@@ -342,7 +342,8 @@ def test_replays_between_calls(call, when):
 
 @pytest.mark.parametrize("ncrit,pack,n", [(64, 0, 1), (64, 0, 33), (64, 0, 65), (33, 0, 500), (64, 1, 3000),
                                           (64, 0, 12000), (48, 1, 20000), (64, 1, (1 << 18) - 3), (32, 1, 17),
-                                          (32, 0, 500), (32, 1, 24), (32, 1, 9000), (24, 1, 30000), (32, 1, 65536)])
+                                          (32, 0, 500), (32, 1, 24), (32, 1, 9000), (24, 1, 30000), (32, 1, 65536),
+                                          (64, 1, 19999), (64, 1, 20000)])
 def test_walk_in_parts(ncrit, pack, n):
     """Groups of 33..64 bodies walked in two parts (up to 2^18 bodies) and of
     17..24 in three (up to 2^16), against block time steps' walk, which has
