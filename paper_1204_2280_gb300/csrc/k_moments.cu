@@ -421,7 +421,7 @@ k_mom_leaves(MomArrays a) {
 // sees every sibling's moments: each sibling's decrement heads a release
 // sequence that this read-modify-write extends).  Only the list's cells
 // start, so a block is not held by climbs for cells that have nothing to do.
-constexpr unsigned MOM_GRAIN = 2, MOM_SPREAD = 1024;
+constexpr unsigned MOM_SPREAD = 1024;
 
 template <bool REFIT>
 __global__ void __launch_bounds__(MOM_CTHREADS, MOM_MINB2)
@@ -436,17 +436,25 @@ k_mom_combine(MomArrays a) {
     __shared__ double s_root[MOM_CTHREADS / 32][10][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned ns = __ldcg(a.nstart);
-    // A warp takes 32 consecutive list entries at a time.  With several
-    // systems they are dealt out in pairs over at least MOM_SPREAD warps, so
-    // that no warp meets many roots (a short list, or small systems' cells at
-    // a list's end).  Moments of 256 systems of 30 bodies in one run / pairs:
-    // 58 / 20 us (each lane its own root, as before: 32), of 64 of 16,384 55 / 52
-    // (single entries 67).  With one system the other warps are better left
-    // idle: dealt out, steps of 2^20 bodies took 0.4% more.
-    constexpr unsigned G = MOM_GRAIN;
-    const unsigned runs = a.multi ? max((ns + 31u) / 32u, min((ns + G - 1u) / G, MOM_SPREAD)) : (ns + 31u) / 32u;
+    // A warp takes 32 list entries at a time: with one system 32 consecutive
+    // ones (dealt out, steps of 2^20 bodies took 0.4% more).  With several
+    // systems they are dealt out over MOM_SPREAD warps in runs of G, as long as
+    // that many warps allow, so that no warp meets many roots (the first
+    // entries are the deepest cells of all systems, and small systems' roots
+    // are in the list themselves).  Multipoles of several systems, us, with
+    // G = 2 / 4 / 8 / 16 / the rule here (in brackets: runs of 32 and each root
+    // by its lane alone):
+    //   256 of 30 bodies      18 /  23 /  33 /  51 /  18   (27)
+    //   256 of 300            27 /  28 /  32 /  38 /  27   (41)
+    //   256 of 4,000          60 /  54 /  51 /  50 /  50   (48)
+    //   256 of 16,000        138 / 122 / 112 / 110 / 107  (108)
+    //    64 of 16,384         54 /  50 /  50 /  50 /  50   (47)
+    //     8 of 200,000        57 /  53 /  51 /  49 /  49   (52)
+    const unsigned lg = a.multi ? min(5u, max(1u, 31u - (unsigned)__clz((int)(ns / MOM_SPREAD) | 1))) : 5u;
+    const unsigned G = 1u << lg;
+    const unsigned runs = max((ns + 31u) / 32u, min((ns + G - 1u) / G, MOM_SPREAD));
     for (unsigned w = blockIdx.x * (MOM_CTHREADS / 32) + warp; w < runs; w += gridDim.x * (MOM_CTHREADS / 32)) {
-        const unsigned j = a.multi ? G * (w + lane / G * runs) + lane % G : w * 32u + lane;
+        const unsigned j = ((w + (lane >> lg) * runs) << lg) + (lane & (G - 1u));
         bool root = false;
         unsigned c = 0u;
         uint2 plk = make_uint2(0u, 0u);

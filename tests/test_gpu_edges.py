@@ -392,7 +392,7 @@ def test_walk_in_parts(ncrit, pack, n):
 
 
 @pytest.mark.parametrize("sizes", [[1], [17], [130], [20000], [30] * 256, [100] * 256, [1, 17, 9000, 16, 600, 2] * 3,
-                                   [17] * 255 + [40000]], ids=lambda s: f"{len(s)}x{s[0]}..{s[-1]}")
+                                   [17] * 255 + [40000], [1500] * 120, [4000] * 200, [17] * 2 + [600000, 500000]], ids=lambda s: f"{len(s)}x{s[0]}..{s[-1]}")
 def test_root_moments(sizes):
     """The roots that a warp combines (none, one or many to a warp) against
     FP64 sums over each system's bodies: sums of at most a hundred FP32 terms
