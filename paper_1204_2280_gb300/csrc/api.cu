@@ -627,10 +627,10 @@ int bonsai_get_bodies(bonsai_ctx *ctx, float *pos, float *vel, int on_device) {
     Ctx tmp = c;   // view with the arrays that hold the state
     tmp.pos4 = (float4 *)P; tmp.vel4 = (float4 *)V; tmp.id = (uint32_t *)I;
     if (on_device) {
-        CK(launch_scatter_bodies(tmp, pos, vel));
+        CK(launch_scatter_bodies(tmp, pos, vel, c.built));
     } else {
         float *sp = c.stage, *sv = c.stage + 3 * c.n;
-        CK(launch_scatter_bodies(tmp, pos ? sp : nullptr, vel ? sv : nullptr));
+        CK(launch_scatter_bodies(tmp, pos ? sp : nullptr, vel ? sv : nullptr, c.built));
         if (pos) CK(cudaMemcpyAsync(pos, sp, 12 * (size_t)c.n, cudaMemcpyDeviceToHost, c.stream));
         if (vel) CK(cudaMemcpyAsync(vel, sv, 12 * (size_t)c.n, cudaMemcpyDeviceToHost, c.stream));
         CK(cudaStreamSynchronize(c.stream));

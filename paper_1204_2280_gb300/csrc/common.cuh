@@ -318,7 +318,7 @@ cudaError_t launch_feature_stats(cudaStream_t s, const float *X, const float *Y,
                                  unsigned *arrived, float *norm);
 cudaError_t launch_kick(Ctx &c, float dt);
 cudaError_t launch_scatter_forces(Ctx &c, float *acc, float *pot);
-cudaError_t launch_scatter_bodies(Ctx &c, float *pos, float *vel);
+cudaError_t launch_scatter_bodies(Ctx &c, float *pos, float *vel, bool sorted);
 cudaError_t launch_scatter_counts(Ctx &c, uint32_t *npc, uint32_t *npp);
 cudaError_t launch_diag(Ctx &c);
 cudaError_t launch_tree_export(Ctx &c, unsigned c0, unsigned cnt, int32_t *bb, int32_t *bc, int32_t *cb,

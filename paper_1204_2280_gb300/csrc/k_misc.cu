@@ -132,9 +132,12 @@ __global__ void k_scatter_bodies(const float4 *__restrict__ pos, const float4 *_
     if (v) { float4 q = vel[i]; v[3 * j] = q.x; v[3 * j + 1] = q.y; v[3 * j + 2] = q.z; }
 }
 
-cudaError_t launch_scatter_bodies(Ctx &c, float *pos, float *vel) {
+// sorted: c.id is the order of a build; before the first one it is the
+// caller's own, the scatter writes whole lines and a gather only adds its
+// first launch (2^18 bodies 8.5 against 5.0 us, 2^22 54 against 41).
+cudaError_t launch_scatter_bodies(Ctx &c, float *pos, float *vel, bool sorted) {
     int n = (int)c.n;
-    if (n >= GATHER_MIN_N && (pos || vel)) {
+    if (sorted && n >= GATHER_MIN_N && (pos || vel)) {
         const cudaError_t e = launch_inverse(c);
         if (e != cudaSuccess) return e;
         k_gather_bodies<<<(n + GATHER_THREADS - 1) / GATHER_THREADS, GATHER_THREADS, 0, c.stream>>>(

@@ -171,6 +171,20 @@ def test_caller_order_outputs(n):
         assert np.array_equal(a2.cpu().numpy(), both[0][perm]) and np.array_equal(p2.cpu().numpy(), both[1][perm])
 
 
+@pytest.mark.parametrize("n", [1, (1 << 18) - 1, (1 << 18) + 1])
+def test_outputs_before_the_first_build(n):
+    """Loaded bodies read back without a build, alone and together."""
+    rng = np.random.default_rng(n)
+    pos, vel = (rng.normal(size=(n, 3)).astype(np.float32) for _ in range(2))
+    with B.Bonsai(B.Config(ncrit=32)) as bz:
+        bz.set_bodies(pos, np.ones(n, np.float32), vel)
+        for want in ((True, True), (True, False), (False, True)):
+            x, v = (np.zeros((n, 3), np.float32) if w else None for w in want)
+            B.bonsai_get_bodies(bz.ctx, x, v)
+            assert (x is None or np.array_equal(x, pos)) and (v is None or np.array_equal(v, vel))
+        bz.sync()
+
+
 @pytest.mark.parametrize("n", [1, 16, 31, 33, 127, 129, 5000])
 def test_network_rows(n):
     """Inference of 32-row warp tiles against the FP64 oracle on the same
