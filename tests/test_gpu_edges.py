@@ -67,7 +67,8 @@ def test_merge_sort_tiles(n):
         assert np.array_equal(out.cpu().numpy(), keys[ref])
 
 
-@pytest.mark.parametrize("n", [1, 4608, 4609, 9217, 36865, (1 << 20) - 1, 1 << 20, (1 << 20) + 1])
+@pytest.mark.parametrize("n", [1, 4608, 4609, 9217, 36865, (1 << 20) - 1, 1 << 20, (1 << 20) + 1, 3000001,
+                               (1 << 22) - 1, 1 << 22, (1 << 22) + 1])
 def test_build_order_across_sorts(n):
     """Keys, permutation and moved bodies of a build on both sides of the
     tile, run and sort choices, with duplicate positions, against the
@@ -90,6 +91,34 @@ def test_build_order_across_sorts(n):
             x, v = np.zeros((n, 3), np.float32), np.zeros((n, 3), np.float32)
             B.bonsai_get_bodies(bz.ctx, x, v)
             assert np.array_equal(x, pos) and np.array_equal(v, pos)
+        bz.sync()
+
+
+def test_build_order_when_the_sort_changes():
+    """One context whose loads cross the sort choice (2^22 bodies) both ways,
+    and that builds several systems in between: the radix sort's counts are
+    its own each time."""
+    import oracle
+    sizes = [(1 << 22) + 1, 70001, (1 << 22) + 3, 4608, 5000]
+    rng = np.random.default_rng(3)
+    pos = rng.normal(size=(max(sizes), 3)).astype(np.float32)
+    mass = np.ones(max(sizes), np.float32)
+    with B.Bonsai(B.Config(ncrit=32)) as bz:
+        for n in sizes:
+            p = pos[-n:]
+            bz.set_bodies(p, mass[:n]).build()
+            k = oracle.keys(p, *oracle.domain(p))
+            ref = _stable(k)
+            kk, pp = B.bonsai_get_keys(bz.ctx)
+            assert np.array_equal(kk, k[ref]) and np.array_equal(pp, ref)
+            if n < 100000:
+                half = n // 3
+                bz.set_bodies(p, mass[:n]).set_systems([0, half, n]).build()
+                kk, pp = B.bonsai_get_keys(bz.ctx)
+                for lo, hi in ((0, half), (half, n)):
+                    k = oracle.keys(p[lo:hi], *oracle.domain(p[lo:hi]))
+                    ref = _stable(k)
+                    assert np.array_equal(kk[lo:hi], k[ref]) and np.array_equal(pp[lo:hi], lo + ref)
         bz.sync()
 
 
