@@ -401,8 +401,8 @@ int bonsai_judge(bonsai_ctx *ctx, float eps, float *p99) {
     if (!c.have_acc) return cfail(ctx, BONSAI_ERR_NOT_READY, "bonsai_judge: no forces yet");
     CCK(launch_judge_targets(c));
     CCK(launch_direct(c, c.judge_targets, c.judge_n, eps, c.judge_partial, JUDGE_SPLIT, c.judge_direct));
-    CCK(launch_judge(c, c.judge_targets, c.judge_n, c.judge_direct, 1e30f));
-    CCK(cudaMemcpyAsync(p99, &c.st->judge_p99, sizeof(float), cudaMemcpyDeviceToHost, c.stream));
+    CCK(launch_judge_own(c, c.judge_targets, c.judge_n, c.judge_direct));
+    CCK(cudaMemcpyAsync(p99, &c.st->own_p99, sizeof(float), cudaMemcpyDeviceToHost, c.stream));
     CCK(cudaStreamSynchronize(c.stream));
     return BONSAI_OK;
 }

@@ -100,6 +100,7 @@ struct DevState {
     unsigned fallback;                // 1: the judge asked for the fine-theta walk
     unsigned judge_tick;              // learned evaluations since the interval was set
     unsigned judge_on;                // 1: this evaluation is judged
+    float own_p99;                    // bonsai_judge's p99
     unsigned long long cyc_active;    // block steps, last cycle: body steps ended (forces taken)
     unsigned long long cyc_inter[2];  // block steps, last cycle: n_pc, n_pp summed over substeps
     unsigned hold_tile;               // testing aid: sort tile hold_tile - 1 never publishes (0: off)
@@ -305,6 +306,7 @@ cudaError_t launch_direct(Ctx &c, const uint32_t *targets, int ntar, float eps, 
                           float4 *out, const unsigned *gate = nullptr);
 cudaError_t launch_judge(Ctx &c, const uint32_t *targets, int ntar, const float4 *direct, float budget,
                          const unsigned *gate = nullptr);
+cudaError_t launch_judge_own(Ctx &c, const uint32_t *targets, int ntar, const float4 *direct);
 cudaError_t launch_mlp_infer(Ctx &c, const float *P, const float *norm);
 cudaError_t launch_mlp_rows(cudaStream_t s, const float *P, const float *norm, const float *X, float *Y, int n);
 cudaError_t launch_mlp_grad(cudaStream_t s, const float *P, const float *norm, const float *X, const float *Y,

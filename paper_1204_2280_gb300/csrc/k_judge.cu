@@ -158,7 +158,7 @@ cudaError_t launch_direct(Ctx &c, const uint32_t *targets, int ntar, float eps, 
 
 // Judge: relative errors |a - a_direct| / |a_direct| at the targets, their
 // 99th percentile (linear interpolation between order statistics, as numpy's
-// default), and the fallback flag p99 > budget.  One block of 1024 threads;
+// default), and the fallback flag p99 > budget (where asked for).  One block of 1024 threads;
 // the two order statistics by bisection on the errors' bits (non-negative
 // floats order as their bits), one block count per bit: 38 us with a bitonic
 // sort of the 4096 errors, 18 us here.  An error that is not finite (forces
@@ -167,7 +167,8 @@ cudaError_t launch_direct(Ctx &c, const uint32_t *targets, int ntar, float eps, 
 // Skipped by the gate, it leaves the last judgement (p99 and flag) in place.
 __global__ void __launch_bounds__(1024)
 k_judge_p99(const float4 *__restrict__ acc4, const uint32_t *__restrict__ targets, int ntar,
-            const float4 *__restrict__ direct, float budget, DevState *st, const unsigned *__restrict__ gate) {
+            const float4 *__restrict__ direct, float budget, float *p99_out, unsigned *fallback,
+            const unsigned *__restrict__ gate) {
     if (gate && *gate == 0u) return;
     constexpr int PER = JUDGE_MAX / 1024;
     __shared__ unsigned s_next;
@@ -209,14 +210,24 @@ k_judge_p99(const float4 *__restrict__ acc4, const uint32_t *__restrict__ target
         const float v0 = __uint_as_float(lo), v1 = tie ? v0 : __uint_as_float(s_next);
         const float f = pos - (float)i0;
         const float p99 = v1 < INFINITY ? v0 + f * (v1 - v0) : f > 0.f ? v1 : v0;
-        st->judge_p99 = p99;
-        st->fallback = p99 <= budget ? 0u : 1u;
+        *p99_out = p99;
+        if (fallback) *fallback = p99 <= budget ? 0u : 1u;
     }
 }
 
+// The judgement of the learned path (p99, fallback by budget; skipped by the
+// gate).
 cudaError_t launch_judge(Ctx &c, const uint32_t *targets, int ntar, const float4 *direct, float budget,
                          const unsigned *gate) {
-    k_judge_p99<<<1, 1024, 0, c.stream>>>(c.acc4, targets, ntar, direct, budget, c.st, gate);
+    k_judge_p99<<<1, 1024, 0, c.stream>>>(c.acc4, targets, ntar, direct, budget, &c.st->judge_p99, &c.st->fallback,
+                                          gate);
+    return cudaGetLastError();
+}
+
+// The p99 of the current accelerations alone: the learned path's judgement
+// stays.
+cudaError_t launch_judge_own(Ctx &c, const uint32_t *targets, int ntar, const float4 *direct) {
+    k_judge_p99<<<1, 1024, 0, c.stream>>>(c.acc4, targets, ntar, direct, 0.f, &c.st->own_p99, nullptr, nullptr);
     return cudaGetLastError();
 }
 

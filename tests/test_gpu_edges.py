@@ -273,6 +273,28 @@ def test_judge_other_bodies(sizes):
         bz.sync()
 
 
+def test_own_judgement_leaves_the_learned_one():
+    """bonsai_judge between learned evaluations: their last judgement (p99 and
+    fallback) stays readable and in force until the next judged one."""
+    n = 3000
+    rng = np.random.default_rng(4)
+    pos, mass = rng.normal(size=(n, 3)).astype(np.float32), np.full(n, 1.0 / n, np.float32)
+    fine, a = np.zeros((n, 3), np.float32), np.zeros((n, 3), np.float32)
+    net = B.MLP(1)
+    with B.Bonsai(B.Config(ncrit=64)) as bz:
+        bz.set_bodies(pos, mass).build().multipoles().forces(0.5, 0.01, fine)
+        B.bonsai_set_learned(bz.ctx, net, 1.0, 0.5, 0.0)         # every judged evaluation falls back
+        B.bonsai_set_judge_interval(bz.ctx, 3)
+        B.bonsai_forces_learned(bz.ctx, 0.01, a)
+        last = B.bonsai_get_judge(bz.ctx)
+        assert last[1] and np.array_equal(a, fine)
+        assert B.bonsai_judge(bz.ctx, 0.01) < last[0]            # of the fine forces, not of the network's
+        assert B.bonsai_get_judge(bz.ctx) == last
+        B.bonsai_forces_learned(bz.ctx, 0.01, a)                 # not judged: the decision holds
+        assert B.bonsai_get_judge(bz.ctx) == last and np.array_equal(a, fine)
+        bz.sync()
+
+
 @pytest.mark.parametrize("n", [1, 300, 5000])
 def test_nan_correction_falls_back(n):
     """A network whose outputs are NaN is rejected by the judge at every finite
