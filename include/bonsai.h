@@ -104,9 +104,9 @@ int bonsai_set_systems(bonsai_ctx *ctx, const long long *offsets, int nsys);
 
 /* Sect. 2 "sorting", "moving", "tree-construction": domain cube, 63-bit
  * Morton keys (21 bits per axis, x in the lowest bit of each triple), stable
- * sort, body reorder, octree (cells with more than nleaf bodies
- * split into their non-empty octants; breadth-first, key order within a
- * level) and walk groups (cells with at most ncrit bodies whose parent has
+ * sort, body reorder, octree (cells with more than nleaf bodies split into
+ * their non-empty octants; breadth-first, key order within a level) and walk
+ * groups (cells with at most ncrit bodies whose parent has
  * more). */
 int bonsai_build(bonsai_ctx *ctx);
 
@@ -240,9 +240,8 @@ int bonsai_set_stage_timing(bonsai_ctx *ctx, int on);
  * ms[0] first kick + drift + domain, [1] keys, [2] sort, [3] reorder (up to
  * 2^22 bodies of one system the sort is a merge sort: [1] then holds the keys
  * and the sort of tiles, [2] the merges, the last of which reorders), [4]
- * tree build, [5] multipoles, [6] walk, [7]
- * second kick.  Synchronises; writes min(n, 8) values and returns that
- * count (negative on error). */
+ * tree build, [5] multipoles, [6] walk, [7] second kick.  Synchronises;
+ * writes min(n, 8) values and returns that count (negative on error). */
 int bonsai_get_stage_times(bonsai_ctx *ctx, float *ms, int n);
 
 /* ---- introspection (copies to caller-owned HOST buffers; synchronises) -- */
@@ -293,9 +292,9 @@ int bonsai_get_counts(bonsai_ctx *ctx, uint32_t *n_pc, uint32_t *n_pp,
  * the merge kernel's shared-memory limit for that device.  Every call reuses
  * the same scratch: calls whose GPU work could overlap (other threads or
  * streams) race and must be serialised by the caller.  Work is ordered on
- * cuda_stream (NULL: the legacy default stream); the call then
- * synchronises that stream, so it cannot run while the stream is being
- * captured into a CUDA graph.  Error text: bonsai_last_error(NULL). */
+ * cuda_stream (NULL: the legacy default stream); the call then synchronises
+ * that stream, so it cannot run while the stream is being captured into a
+ * CUDA graph.  Error text: bonsai_last_error(NULL). */
 int bonsai_sort_keys_static(const uint64_t *keys, uint64_t *sorted_keys,
                             uint32_t *perm, long long n, void *cuda_stream);
 
@@ -381,7 +380,9 @@ int bonsai_learn_samples(bonsai_ctx *ctx, float theta, float eps, int ntar, unsi
 /* Judge of the current accelerations: direct sum (FP32 tiles and a FP32
  * reduction over source splits, both Kahan-compensated) at min(n, 4096)
  * bodies spaced evenly in key order and the 99th
- * percentile (numpy's linear interpolation) of |a - a_direct| / |a_direct|. */
+ * percentile (numpy's linear interpolation) of |a - a_direct| / |a_direct|;
+ * errors that are not finite rank as infinite.  The learned path's last
+ * judgement (bonsai_get_judge) stays. */
 int bonsai_judge(bonsai_ctx *ctx, float eps, float *p99);
 
 /* Use the learned correction in bonsai_step and bonsai_forces_learned: walk

@@ -414,7 +414,8 @@ int bonsai_multipoles(bonsai_ctx *ctx) {
     const bool reset = !seen_capture(c) && !c.have_acc;
     c.walk_ready = false;
     const long long key[] = {c.n, c.arena_gen, c.nsys, c.cells_hint, reset};
-    CK(run_cached(c, c.mom_graph, key, (int)(sizeof key / sizeof key[0]), [&]() { return launch_multipoles(c, reset); }));
+    CK(run_cached(c, c.mom_graph, key, (int)(sizeof key / sizeof key[0]),
+                  [&]() { return launch_multipoles(c, reset); }));
     c.walk_ready = reset;
     c.moments_ready = true;
     return BONSAI_OK;

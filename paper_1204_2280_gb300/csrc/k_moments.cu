@@ -507,8 +507,8 @@ static unsigned multipole_blocks(const Ctx &c) {
 }
 
 static MomArrays mom_arrays(Ctx &c, bool refit, bool reset) {
-    return MomArrays{c.st, reset ? c.st : nullptr, c.cell_body, c.cell_link, c.cell_level, c.cell_parent, c.cell_done, c.pos4, c.keys,
-                     c.sysid, c.mono, c.quadA, c.quadB, c.delta, refit ? c.cext : nullptr, c.nsys > 1,
+    return MomArrays{c.st, reset ? c.st : nullptr, c.cell_body, c.cell_link, c.cell_level, c.cell_parent, c.cell_done,
+                     c.pos4, c.keys, c.sysid, c.mono, c.quadA, c.quadB, c.delta, refit ? c.cext : nullptr, c.nsys > 1,
                      c.cell_start, &c.st->mom_starts};
 }
 

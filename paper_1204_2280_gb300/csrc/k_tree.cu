@@ -13,10 +13,10 @@
 // launches: (1) per body, the levels on which it starts cells and its group,
 // compacted per block into a list of the bodies that start any (about one per
 // leaf), with counts per block and level; (2) scan of those counts over the
-// blocks (small trees: pass 3 adds them up); (3) per listed body, the index, first body, level and link of each
-// of its cells and its groups; (4) child counts and parents.  Internal
-// cells' body counts, which no stage of a step reads, are derived on demand
-// for the tree getter (k_internal_counts).
+// blocks (small trees: pass 3 adds them up); (3) per listed body, the index,
+// first body, level and link of each of its cells and its groups; (4) child
+// counts and parents.  Internal cells' body counts, which no stage of a step
+// reads, are derived on demand for the tree getter (k_internal_counts).
 #include "common.cuh"
 
 namespace bonsai {
@@ -267,7 +267,8 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
         const unsigned et = S.e_t[e], ed = S.e_d[e];
         const int elo = (int)(ed & 0xffu), ehi = (int)((ed >> 8) & 0xffu), elg = (int)((ed >> 16) & 0xffu);
         const int kind = (int)(ed >> 24);
-        const int lend = e + 1 < ne ? (int)S.e_t[e + 1] : run_end_local(S, k0, base, (int)et, ehi, n, sk, st, sysid, multi);
+        const int lend = e + 1 < ne ? (int)S.e_t[e + 1]
+                                    : run_end_local(S, k0, base, (int)et, ehi, n, sk, st, sysid, multi);
         const unsigned lcnt = (unsigned)lend - et;
         unsigned gcnt = 0u, ngrp = 0u;
         if (kind == 1) {
@@ -276,7 +277,8 @@ k_build_mark(const unsigned long long *__restrict__ sk, const uint8_t *__restric
             } else {
                 unsigned j = e + 1;
                 while (j < ne && (S.e_d[j] & 0xffu) > (unsigned)elg) j++;
-                const int gend = j < ne ? (int)S.e_t[j] : run_end_local(S, k0, base, (int)et, elg, n, sk, st, sysid, multi);
+                const int gend = j < ne ? (int)S.e_t[j]
+                                        : run_end_local(S, k0, base, (int)et, elg, n, sk, st, sysid, multi);
                 gcnt = (unsigned)gend - et;
             }
             ngrp = 1u;

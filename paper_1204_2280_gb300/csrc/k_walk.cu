@@ -637,7 +637,8 @@ size_t walk_smem_bytes(int warps, int stack_cap) {
 // Function attribute and occupancy are set up once per shape, before any
 // stream capture of a step (the first step always runs eagerly).
 template <int BPL, bool FEAT, bool BLOCK, int SPLIT = 0>
-static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned *gate, bool three, cudaStream_t stream) {
+static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned *gate, bool three,
+                                 cudaStream_t stream) {
     const unsigned polls = (unsigned)(c.max_spin < 0xffffffffll ? c.max_spin : 0xffffffffll);
     const int warps = c.walk_warps;
     const size_t smem = walk_smem_bytes(warps, c.list_capacity);
@@ -651,7 +652,8 @@ static cudaError_t launch_walk_t(Ctx &c, float theta, float eps, const unsigned 
     if (dv < 0 || dv >= MAX_DEVICES) return cudaErrorInvalidDevice;
     if (occ_warps[dv] != warps || occ_smem[dv] != smem) {
         int per = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<BPL, FEAT, BLOCK, SPLIT>, warps * 32, smem);
+        cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<BPL, FEAT, BLOCK, SPLIT>, warps * 32, smem);
         if (e != cudaSuccess) return e;
         occ_warps[dv] = warps; occ_smem[dv] = smem; occ_per_sm[dv] = per < 1 ? 1 : per;
     }
@@ -744,7 +746,7 @@ cudaError_t launch_walk(Ctx &c, float theta, float eps, bool features, const uns
 // The group walk with another opening rule and kernel: a cell is searched
 // iff its cube (build-time centre, half side ext) comes within h_max of the
 // group's box, h_max the largest smoothing length of the group; searched
-// leaves feed their bodies through a ring of 64 in shared memory; each body
+// leaves feed their bodies through a ring in shared memory; each body
 // i counts the sources j with r^2 < h_i^2 (r^2 = fma(dz, dz, fma(dy, dy,
 // dx dx)), dx = x_j - x_i rounded: the decision the oracle takes) and sums
 // m_j W(r, h_i), W the cubic spline of compact support h.  Up to 64 bodies
